@@ -25,9 +25,10 @@
 //   2b/(1+q) (b/R)^(t-1) e^{i phi} e^{i phi_ell} = (thetaE/rho)^t w
 // (b = thetaE sqrt(q), R = sqrt(q) rho) have been applied. It is smooth in
 // (e1, e2) through e = 0, needs no atan2 and no rotation, and gives the
-// gradient with respect to e1, e2 in closed form. G is evaluated by Horner's
-// rule on the coefficients a_1..a_N (per-vector term count N, so all rays of
-// a vector run the same loop): one complex multiply-add per term.
+// gradient with respect to e1, e2 in closed form. The sum runs over the
+// coefficients a_1..a_N (per-vector term count N, so all rays of a vector run
+// the same loop), by Horner's rule on G (one complex multiply-add per term)
+// or by the second-order recurrence of epl_fwd_T (two FMAs per term).
 //
 // The Sersic profile (Eq. Sersic) uses the same quadratic form for its
 // elliptical radius: q x_l^2 + y_l^2 / q = A dx^2 + 2 B dx dy + C dy^2 with
@@ -59,11 +60,11 @@ constexpr float RHO2_MIN = 1e-12f;   // (1e-6 arcsec)^2: EPL deflection zero / S
 constexpr int RAY_THREADS = 256;     // block size of the ray kernels
 constexpr int FINAL_THREADS = 128;   // block size of k_final (vectors per block)
 
-// Accumulator slots of the adjoint (per vector, before the chain rule).
+// Accumulator slots of the adjoint (per vector, before the chain rule; see
+// ray_adj and light_adj for what each sums).
 enum Acc {
-  A_THETAE = 0, A_T, A_E1, A_E2, A_XC, A_YC, A_G1, A_G2,            // mass (x b_s/n_s)
-  A_L_R, A_L_N1, A_L_N2, A_L_E1, A_L_E2, A_L_X, A_L_Y, A_L_I,        // lens light
-  A_S_R, A_S_N1, A_S_N2, A_S_E1, A_S_E2, A_S_X, A_S_Y, A_S_I         // source
+  A_THETAE = 0, A_T, A_E1, A_E2, A_QR, A_QI, A_G1, A_G2,   // mass (x b_s/n_s I_s)
+  A_L = 8, A_S = 16                                        // eight moments each of the lens light and the source
 };
 
 struct LightC {
@@ -86,17 +87,19 @@ struct __align__(16) VecConst {
   float w2min;             // RHO2_MIN (1 - |eps|^2): |w|^2 below it is rho < 1e-6 arcsec
   float g1, g2;            // external shear
   int nterms;              // series terms of F (0 <= N <= NMAX); < 0 marks an invalid vector
-  int nterms_adj;          // series terms in the adjoint, max(N, 1)
+  int npairs;              // pairs of terms the ray loops sum, ceil(max(N, 1) / 2)
   float th;                // t / 2
   float kc;                // 1 - t/2, for dF/du = [(t/2) F - (1 - t/2) G] / (1 - u)
-  float kap_c;             // (2 - t) / 2: kappa = kap_c (thetaE/rho)^t
+  float u2;                // |u|^2 = |eps|^2 of every ray
   float omt;               // 1 - t
   float e1i, e2i;          // e1, e2 times 1 / (1 - |eps|^2)
   int order;               // written by k_order into slot p: the vector the ray kernels take p-th
-  float pad_[3];
+  float den0;              // 1 + |eps|^2: |1 - u|^2 = den0 - 2 Re u
+  float pad_[2];
   LightC light[2];         // [0] lens light at theta, [1] source at beta
-  float an[NMAX];          // a_n = c_1 ... c_n, n = 1..NMAX at index n-1
-  float ant[NMAX];         // d a_n / d t
+  // the series two terms at a time: (a_{2m+1}, a_{2m+2}, b_{2m+1}, b_{2m+2}), a_n = c_1 ... c_n and
+  // b_n = d a_n / d t / ln 2, zero past the term count
+  float4 ser[NMAX / 2];
 };
 static_assert(sizeof(VecConst) % 16 == 0, "VecConst must be a whole number of 16-byte words");
 
@@ -198,7 +201,13 @@ struct F2 {
 __device__ __forceinline__ F2 operator+(F2 a, F2 b) { return {__fadd2_rn(a.v, b.v)}; }
 __device__ __forceinline__ F2 operator*(F2 a, F2 b) { return {__fmul2_rn(a.v, b.v)}; }
 __device__ __forceinline__ F2 operator-(F2 a, F2 b) { return {__ffma2_rn(b.v, make_float2(-1.f, -1.f), a.v)}; }
-__device__ __forceinline__ F2 operator-(F2 a) { return {__fmul2_rn(a.v, make_float2(-1.f, -1.f))}; }
+// Sign flip on the integer pipe: the ray kernels are bound by the FP32 pipe,
+// and packed instructions take no negated operands (k_ray_adj at 60 x 60,
+// k = 2, B = 4096: 459 -> 452 us against a packed multiply by -1).
+__device__ __forceinline__ F2 operator-(F2 a) {
+  return {make_float2(__uint_as_float(__float_as_uint(a.v.x) ^ 0x80000000u),
+                      __uint_as_float(__float_as_uint(a.v.y) ^ 0x80000000u))};
+}
 
 template <class T> __device__ __forceinline__ T sp(float a);
 template <> __device__ __forceinline__ float sp<float>(float a) { return a; }
@@ -247,21 +256,62 @@ __device__ __forceinline__ F2 lg2cT(F2 a) {
 // adds instead of converting an integer per ray.
 __device__ __forceinline__ F2 grid_coord2(F2 n, float hh, float hl) { return fmaT(n, sp<F2>(hh), n * sp<F2>(hl)); }
 
+// ------------------------------------------------------- ray constants ---
+// What the ray loops read of a vector's VecConst, as values the compiler
+// knows to be the same in every lane of the warp (a shuffle from lane 0), so
+// that it can hold them in uniform registers: copied from shared memory into
+// ordinary ones they took 31 registers of every thread, and with the 24 packed
+// accumulators the adjoint then fitted three blocks per SM with spills
+// (k_ray_adj at 60 x 60, k = 2, B = 4096: 448.5 -> 428 us at three blocks, and
+// 406 us at the four that fit with them).
+struct RayLight {
+  float A, B2, C, x, y, c1, r2min, k1, I0;
+};
+struct RayC {
+  float xc, yc, e1, e2, lc, tlc_lo, t, w2min, g1, g2, th, kc, u2, omt, den0;
+  int npairs;
+  RayLight light[2];
+};
+__device__ __forceinline__ float warp_uniform(float v) { return __shfl_sync(0xffffffffu, v, 0); }
+__device__ __forceinline__ int warp_uniform(int v) { return __shfl_sync(0xffffffffu, v, 0); }
+__device__ __forceinline__ RayLight ray_light(const LightC& l) {
+  return {warp_uniform(l.A),  warp_uniform(l.B2),    warp_uniform(l.C),  warp_uniform(l.x), warp_uniform(l.y),
+          warp_uniform(l.c1), warp_uniform(l.r2min), warp_uniform(l.k1), warp_uniform(l.I0)};
+}
+__device__ __forceinline__ RayC ray_consts(const VecConst& v) {
+  return {warp_uniform(v.xc), warp_uniform(v.yc),     warp_uniform(v.e1), warp_uniform(v.e2),
+          warp_uniform(v.lc), warp_uniform(v.tlc_lo), warp_uniform(v.t),  warp_uniform(v.w2min),
+          warp_uniform(v.g1), warp_uniform(v.g2),     warp_uniform(v.th), warp_uniform(v.kc),
+          warp_uniform(v.u2), warp_uniform(v.omt),    warp_uniform(v.den0), warp_uniform(v.npairs),
+          {ray_light(v.light[0]), ray_light(v.light[1])}};
+}
+
 // Elliptical Sersic at (px, py), generic in the ray type; the forward model,
 // so its log2 is the unbiased one (log L sums the model over every pixel).
+// The terms of dy alone come first: the ray loops step x innermost, so the
+// compiler can keep the lens light's out of the inner loop.
 template <class T>
-__device__ __forceinline__ T sersic_fwd_T(const LightC& L, T px, T py) {
+__device__ __forceinline__ T sersic_fwd_T(const RayLight& L, T px, T py) {
   const T dx = px - sp<T>(L.x), dy = py - sp<T>(L.y);
-  T r2 = fmaT(sp<T>(L.A) * dx, dx, fmaT(sp<T>(L.B2) * dx, dy, sp<T>(L.C) * dy * dy));
+  T r2 = fmaT(fmaT(sp<T>(L.A), dx, sp<T>(L.B2) * dy), dx, sp<T>(L.C) * dy * dy);
   r2 = maxT(r2, sp<T>(L.r2min));
   const T s = ex2T(sp<T>(L.c1) * lg2cT(r2));
   return sp<T>(L.I0) * ex2T(fmaT(sp<T>(-L.k1), s, sp<T>(L.k1)));
 }
 
+// Series of at most 26 terms (|eps| up to about 0.5) are summed by
+// the second-order recurrence for a real polynomial at a complex point
+// (Knuth, TAOCP 4.6.4; |u|^2 = |eps|^2 for every ray): two FMAs a term
+// instead of Horner's four. Its error against 64 bits over |u| = f is
+// Horner's at f <= 0.5 (rms 3.2e-8, max 1.0e-7 for both), above it grows with
+// 1 / (1 - f)^2 (f = 0.7: max 2.4e-7 against 1.1e-7; f = 0.85: 1.0e-6 against
+// 1.4e-7), so longer series keep Horner's rule.
+constexpr int RECURRENCE_MAX_PAIRS = 13;
+
 // EPL deflection, generic in the ray type. A ray inside rho < 1e-6 arcsec gets
 // zero deflection (mask), computed without a branch so pairs stay in lockstep.
 template <class T>
-__device__ __forceinline__ void epl_fwd_T(const VecConst& V, const float* an, T x, T y, T& ax, T& ay) {
+__device__ __forceinline__ void epl_fwd_T(const RayC& V, const float4* ser, T x, T y, T& ax, T& ay) {
   const T dx = x - sp<T>(V.xc), dy = y - sp<T>(V.yc);
   // w = z - eps conj(z) = (dx - e1 dx - e2 dy, dy + e1 dy - e2 dx)
   const T wr = fmaT(sp<T>(-V.e1), dx, fmaT(sp<T>(-V.e2), dy, dx));
@@ -270,34 +320,74 @@ __device__ __forceinline__ void epl_fwd_T(const VecConst& V, const float* an, T 
   const T keep = geT(w2, sp<T>(V.w2min));
   const T w2c = maxT(w2, sp<T>(V.w2min));   // > 0; where it clamps, keep = 0 zeroes the deflection
   const T S = keep * ex2T(fmaT(sp<T>(V.t), fmaT(sp<T>(-0.5f), lg2T(w2c), sp<T>(V.lc)), sp<T>(V.tlc_lo)));
-  const T iw2 = rcpT(w2c);
-  const T nwi = -wi;
-  const T vr = fmaT(wr, wr, nwi * wi) * iw2;
-  const T vi = sp<T>(2.f) * wr * wi * iw2;
-  const T ur = fmaT(sp<T>(-V.e1), vr, sp<T>(-V.e2) * vi);
-  const T ui = fmaT(sp<T>(V.e2), vr, sp<T>(-V.e1) * vi);
-  const T nui = fmaT(sp<T>(-V.e2), vr, sp<T>(V.e1) * vi);   // -ui: packed FMAs take no negated operands
-  // G = sum_{n<N} a_{n+1} u^n by Horner (g = a_n + u g), then F = 1 + u G
-  T gr = sp<T>(0.f), gi = sp<T>(0.f);
-#pragma unroll 2
-  for (int n = V.nterms; n >= 1; --n) {
-    const T ngr = fmaT(ur, gr, fmaT(nui, gi, sp<T>(an[n - 1])));
-    gi = fmaT(ur, gi, ui * gr);
-    gr = ngr;
+  // v = w / conj(w) = (1 - 2 wi^2 / |w|^2, 2 wr wi / |w|^2), u = -conj(eps) v
+  const T nm = sp<T>(-2.f) * rcpT(w2c) * wi;
+  const T vr = fmaT(wi, nm, sp<T>(1.f)), nvi = wr * nm;
+  const T ur = fmaT(sp<T>(-V.e1), vr, sp<T>(V.e2) * nvi);
+  const T ui = fmaT(sp<T>(V.e2), vr, sp<T>(V.e1) * nvi);
+  // F = 1 + sum_n a_n u^n; the two highest terms start the sum (the table is
+  // zero past the term count), then two more per step
+  T hr, hi;
+  const float4 top = ser[V.npairs - 1];
+  if (V.npairs <= RECURRENCE_MAX_PAIRS) {
+    const T ru = ur + ur, nu2 = sp<T>(-V.u2);
+    T c2 = sp<T>(top.y), c1 = fmaT(ru, c2, sp<T>(top.x));
+    for (int m = V.npairs - 2; m >= 0; --m) {
+      const float2 q = *reinterpret_cast<const float2*>(&ser[m]);
+      c2 = fmaT(ru, c1, fmaT(nu2, c2, sp<T>(q.y)));
+      c1 = fmaT(ru, c2, fmaT(nu2, c1, sp<T>(q.x)));
+    }
+    hr = fmaT(ur, c1, fmaT(nu2, c2, sp<T>(1.f)));
+    hi = ui * c1;
+  } else {
+    // G = sum a_{n+1} u^n by Horner (g = a_n + u g), then F = 1 + u G
+    const T nui = -ui;
+    T gr = fmaT(ur, sp<T>(top.y), sp<T>(top.x)), gi = ui * sp<T>(top.y);
+    for (int m = V.npairs - 2; m >= 0; --m) {
+      const float2 q = *reinterpret_cast<const float2*>(&ser[m]);
+      const T n1 = fmaT(ur, gr, fmaT(nui, gi, sp<T>(q.y)));
+      gi = fmaT(ur, gi, ui * gr);
+      const T n0 = fmaT(ur, n1, fmaT(nui, gi, sp<T>(q.x)));
+      gi = fmaT(ur, gi, ui * n1);
+      gr = n0;
+    }
+    hr = fmaT(ur, gr, fmaT(nui, gi, sp<T>(1.f)));
+    hi = fmaT(ur, gi, ui * gr);
   }
-  const T hr = fmaT(ur, gr, fmaT(nui, gi, sp<T>(1.f)));
-  const T hi = fmaT(ur, gi, ui * gr);
-  ax = S * fmaT(wr, hr, nwi * hi);
+  ax = S * fmaT(wr, hr, -(wi * hi));
   ay = S * fmaT(wr, hi, wi * hr);
 }
 
+// Source-plane position of a ray: lens equation with external shear.
 template <class T>
-__device__ __forceinline__ T ray_intensity_T(const VecConst& V, const float* an, T x, T y) {
+__device__ __forceinline__ void source_position_T(const RayC& V, const float4* ser, T x, T y, T& bx, T& by) {
   T ax, ay;
-  epl_fwd_T(V, an, x, y, ax, ay);
-  const T bx = x - ax - fmaT(sp<T>(V.g1), x, sp<T>(V.g2) * y);
-  const T by = y - ay - fmaT(sp<T>(V.g2), x, sp<T>(-V.g1) * y);
+  epl_fwd_T(V, ser, x, y, ax, ay);
+  bx = x - ax - fmaT(sp<T>(V.g1), x, sp<T>(V.g2) * y);
+  by = y - ay - fmaT(sp<T>(V.g2), x, sp<T>(-V.g1) * y);
+}
+
+template <class T>
+__device__ __forceinline__ T ray_intensity_T(const RayC& V, const float4* ser, T x, T y) {
+  T bx, by;
+  source_position_T(V, ser, x, y, bx, by);
   return sersic_fwd_T(V.light[1], bx, by) + sersic_fwd_T(V.light[0], x, y);
 }
+
+// A thread's pixel p and its row i and column j, stepped by a fixed number of
+// pixels without a division per step (two divisions per pixel pair were about
+// a tenth of the forward kernel's instructions at k = 2).
+struct PixelStep {
+  int di, dj;   // rows and columns of a step
+  __device__ __forceinline__ PixelStep(int step, int W) : di(step / W), dj(step - di * W) {}
+  __device__ __forceinline__ void advance(int& i, int& j, int W) const {
+    i += di;
+    j += dj;
+    if (j >= W) {
+      j -= W;
+      ++i;
+    }
+  }
+};
 
 }  // namespace gl

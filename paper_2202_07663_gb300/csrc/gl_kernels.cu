@@ -256,9 +256,10 @@ __device__ __forceinline__ int term_count(int lane, float t, float f, float lf, 
 
 // a_n = c_1 ... c_n and d a_n / d t for n <= 32 NC by a warp scan of the pairs
 // (c_k, d c_k / d t) under (x1, y1) (x2, y2) = (x1 x2, x1 y2 + x2 y1) (the
-// product rule); the first chunk's values do not depend on NC.
+// product rule); the first chunk's values do not depend on NC. Terms past
+// nterms are stored as zero: the ray loops sum them in pairs.
 template <int NC>
-__device__ __forceinline__ void series_coeffs(int lane, float t, VecConst* V) {
+__device__ __forceinline__ void series_coeffs(int lane, float t, int nterms, VecConst* V) {
   float xs[NC], ys[NC];
 #pragma unroll
   for (int m = 0; m < NC; ++m) {
@@ -280,8 +281,10 @@ __device__ __forceinline__ void series_coeffs(int lane, float t, VecConst* V) {
 #pragma unroll
   for (int m = 0; m < NC; ++m) {
     const float x = tx * xs[m], y = fmaf(tx, ys[m], xs[m] * ty);
-    V->an[lane + 32 * m] = x;
-    V->ant[lane + 32 * m] = y;
+    const int n = lane + 32 * m;   // term n + 1
+    float* q = reinterpret_cast<float*>(&V->ser[n >> 1]) + (n & 1);
+    q[0] = n < nterms ? x : 0.f;
+    q[2] = n < nterms ? 1.44269504088896341f * y : 0.f;   // over ln 2, as the adjoint accumulates it
     tx = __shfl_sync(0xffffffffu, x, 31);
     ty = __shfl_sync(0xffffffffu, y, 31);
   }
@@ -340,8 +343,9 @@ __global__ void k_setup(const __grid_constant__ Src src) {
       V->g2 = pp[7];
       V->th = 0.5f * t;
       V->kc = 1.f - 0.5f * t;
-      V->kap_c = 0.5f * (2.f - t);
       V->omt = 1.f - t;
+      V->u2 = e2s;
+      V->den0 = 1.f + e2s;
       V->e1i = e1 * i1me2;
       V->e2i = e2 * i1me2;
     } else if (lane == 1 || lane == 2) {
@@ -356,14 +360,14 @@ __global__ void k_setup(const __grid_constant__ Src src) {
     const float ltol = logf(float(SERIES_TOL));
     int n_fwd = term_count<1>(lane, t, f, lf, ltol);
     if (n_fwd < 32) {   // warp-uniform
-      series_coeffs<1>(lane, t, V);
+      series_coeffs<1>(lane, t, max(n_fwd, 1), V);
     } else {
       n_fwd = term_count<NMAX / 32>(lane, t, f, lf, ltol);
-      series_coeffs<NMAX / 32>(lane, t, V);
+      series_coeffs<NMAX / 32>(lane, t, min(n_fwd, NMAX), V);
     }
     if (lane == 0) {
       V->nterms = ok ? min(n_fwd, NMAX) : -1;
-      V->nterms_adj = max(min(n_fwd, NMAX), 1);
+      V->npairs = (max(min(n_fwd, NMAX), 1) + 1) >> 1;
     }
   }
 }
@@ -516,16 +520,17 @@ __global__ void __launch_bounds__(ORDER_THREADS) k_order(const __grid_constant__
 
 // ----------------------------------------------------------- k_ray_fwd ----
 
-#ifndef GL_FWD_THREADS
-#define GL_FWD_THREADS 128
-#endif
-#ifndef GL_FWD_MINB
-#define GL_FWD_MINB 4
-#endif
-constexpr int FWD_THREADS = GL_FWD_THREADS;
+// Block size and resident blocks per SM of the forward kernel. It is bound by
+// issue slots and the FP32 pipe together (65% and 62% busy). At 60 x 60, k = 2,
+// B = 4096, blocks of 128 threads: four per SM (105 registers) 211 us, five
+// (95) 198, six (80, 52 bytes of spills) 201, seven 205; 244 us before the
+// series went from Horner's rule to the second-order recurrence, the
+// constants became warp-uniform and the divisions left the pixel loop.
+constexpr int FWD_THREADS = 128;
+constexpr int FWD_BLOCKS_PER_SM = 5;
 
 template <class Src>
-__global__ void __launch_bounds__(FWD_THREADS, GL_FWD_MINB) k_ray_fwd(const __grid_constant__ Src src) {
+__global__ void __launch_bounds__(FWD_THREADS, FWD_BLOCKS_PER_SM) k_ray_fwd(const __grid_constant__ Src src) {
   __shared__ VecConst sv;
   __shared__ Seg ss;
   const PdlScope pdl;
@@ -544,15 +549,16 @@ __global__ void __launch_bounds__(FWD_THREADS, GL_FWD_MINB) k_ray_fwd(const __gr
     const int p1 = min(HW, p0 + ss.tile_pix);
     const float inv_k2 = 1.0f / float(k * k);
     const bool valid = sv.nterms >= 0;
+    const RayC rc = ray_consts(sv);
     float* out = ss.work + size_t(b) * HW;
     // two pixels per thread and step (p and p + blockDim), their rays paired in f32x2
     const int stride = blockDim.x;
-    for (int p = p0 + threadIdx.x; p < p1; p += 2 * stride) {
-      const int q = p + stride;
+    const PixelStep step(2 * stride, W);
+    int ip = (p0 + int(threadIdx.x)) / W, jp = p0 + int(threadIdx.x) - ip * W;
+    int iq = (p0 + int(threadIdx.x) + stride) / W, jq = p0 + int(threadIdx.x) + stride - iq * W;
+    for (int p = p0 + threadIdx.x; p < p1; p += 2 * stride, step.advance(ip, jp, W), step.advance(iq, jq, W)) {
+      const int q = p + stride;   // past the tile: its rays are computed and not stored
       const bool has_q = q < p1;
-      const int qq = has_q ? q : p;
-      const int ip = p / W, jp = p - ip * W;
-      const int iq = qq / W, jq = qq - iq * W;
       F2 acc = sp<F2>(0.f);
       if (valid) {
         // grid indices of the pixels' first subpixels; a subpixel step adds 2
@@ -564,7 +570,7 @@ __global__ void __launch_bounds__(FWD_THREADS, GL_FWD_MINB) k_ray_fwd(const __gr
           F2 nx = nx0;
           for (int c = 0; c < k; ++c, nx = nx + sp<F2>(2.f)) {
             const F2 x = grid_coord2(nx, ss.hh, ss.hl);
-            acc = acc + ray_intensity_T(sv, sv.an, x, y);
+            acc = acc + ray_intensity_T(rc, sv.ser, x, y);
           }
         }
         acc = acc * sp<F2>(inv_k2);
@@ -584,7 +590,7 @@ __global__ void __launch_bounds__(FWD_THREADS, GL_FWD_MINB) k_ray_fwd(const __gr
 // ray pass (both share the rays, the source the deflection); the vector's own
 // amplitudes are not used. Invalid vectors get NaN in both slots.
 template <class Src>
-__global__ void __launch_bounds__(FWD_THREADS, GL_FWD_MINB) k_ray_fwd_basis(const __grid_constant__ Src src) {
+__global__ void __launch_bounds__(FWD_THREADS, FWD_BLOCKS_PER_SM) k_ray_fwd_basis(const __grid_constant__ Src src) {
   __shared__ VecConst sv;
   __shared__ Seg ss;
   const PdlScope pdl;
@@ -598,11 +604,8 @@ __global__ void __launch_bounds__(FWD_THREADS, GL_FWD_MINB) k_ray_fwd_basis(cons
     block_copy(&sv, ss.vc + q);
     __syncthreads();
     const int b = ss.ray_order ? slot_checked(sv.order, q, ss.B) : q;   // the vector in slot q
-    if (threadIdx.x == 0) {
-      sv.light[0].I0 = 1.f;
-      sv.light[1].I0 = 1.f;
-    }
-    __syncthreads();
+    RayC rc = ray_consts(sv);
+    rc.light[0].I0 = rc.light[1].I0 = 1.f;
     const int HW = ss.H * ss.W, W = ss.W, k = ss.k;
     const int p0 = tile * ss.tile_pix;
     const int p1 = min(HW, p0 + ss.tile_pix);
@@ -611,12 +614,12 @@ __global__ void __launch_bounds__(FWD_THREADS, GL_FWD_MINB) k_ray_fwd_basis(cons
     float* out_l = ss.work + size_t(2 * b) * HW;
     float* out_s = out_l + HW;
     const int stride = blockDim.x;
-    for (int p = p0 + threadIdx.x; p < p1; p += 2 * stride) {
-      const int q = p + stride;
+    const PixelStep step(2 * stride, W);
+    int ip = (p0 + int(threadIdx.x)) / W, jp = p0 + int(threadIdx.x) - ip * W;
+    int iq = (p0 + int(threadIdx.x) + stride) / W, jq = p0 + int(threadIdx.x) + stride - iq * W;
+    for (int p = p0 + threadIdx.x; p < p1; p += 2 * stride, step.advance(ip, jp, W), step.advance(iq, jq, W)) {
+      const int q = p + stride;   // past the tile: its rays are computed and not stored
       const bool has_q = q < p1;
-      const int qq = has_q ? q : p;
-      const int ip = p / W, jp = p - ip * W;
-      const int iq = qq / W, jq = qq - iq * W;
       F2 acc_l = sp<F2>(0.f), acc_s = sp<F2>(0.f);
       if (valid) {
         const F2 ny0 = {make_float2(float(2 * ip * k + ss.ny0), float(2 * iq * k + ss.ny0))};
@@ -627,12 +630,10 @@ __global__ void __launch_bounds__(FWD_THREADS, GL_FWD_MINB) k_ray_fwd_basis(cons
           F2 nx = nx0;
           for (int c = 0; c < k; ++c, nx = nx + sp<F2>(2.f)) {
             const F2 x = grid_coord2(nx, ss.hh, ss.hl);
-            F2 ax, ay;
-            epl_fwd_T(sv, sv.an, x, y, ax, ay);
-            const F2 bx = x - ax - fmaT(sp<F2>(sv.g1), x, sp<F2>(sv.g2) * y);
-            const F2 by = y - ay - fmaT(sp<F2>(sv.g2), x, sp<F2>(-sv.g1) * y);
-            acc_s = acc_s + sersic_fwd_T(sv.light[1], bx, by);
-            acc_l = acc_l + sersic_fwd_T(sv.light[0], x, y);
+            F2 bx, by;
+            source_position_T(rc, sv.ser, x, y, bx, by);
+            acc_s = acc_s + sersic_fwd_T(rc.light[1], bx, by);
+            acc_l = acc_l + sersic_fwd_T(rc.light[0], x, y);
           }
         }
         acc_l = acc_l * sp<F2>(inv_k2);
@@ -653,47 +654,76 @@ __global__ void __launch_bounds__(FWD_THREADS, GL_FWD_MINB) k_ray_fwd_basis(cons
 
 // ---------------------------------------------------------- k_ray_adj -----
 
-// Lens or source light: accumulates R, n (two terms), e1, e2, x, y, I0 slots
-// and returns (Gx, Gy) = s I / rho^2 (A dx + B dy, B dx + C dy), so that
-// dI/d(centre) = (b_n/n) (Gx, Gy) and dI/d(position) = -(b_n/n) (Gx, Gy).
-// Generic in the ray type (float or a packed pair).
+// Moments of one light profile (lens or source) of a ray at (px, py) with
+// weight g, for I0 = 1 (k_final multiplies by the amplitude):
+//   acc[0] g e s          (e = exp2(k1 (1 - s)), s = (rho^2 / R_eff^2)^c1)
+//   acc[1] g e s log2 s
+//   acc[2], acc[3]        gq dx, gq dy,  gq = g e s R_eff^2 / rho^2 (0 where the radius is floored)
+//   acc[4 .. 6]           gq dx^2, gq dx dy, gq dy^2
+//   acc[7] g e
+// The profile's eight derivatives are linear in these with coefficients that
+// every ray of a vector shares (A, B, C and their derivatives in e1, e2), so
+// k_final forms them once per vector instead of each ray. Returns gq dx and
+// gq dy: (A qx + B qy, B qx + C qy) is the ray's position derivative over
+// -(b_n / n) I0. Generic in the ray type (float or a packed pair).
 template <class T>
-__device__ __forceinline__ void light_adj(const LightC& L, T px, T py, T g, T* acc, T& Gx, T& Gy) {
+__device__ __forceinline__ void light_adj(const RayLight& L, T px, T py, T g, T* acc, T& qx, T& qy) {
   const T dx = px - sp<T>(L.x), dy = py - sp<T>(L.y);
-  const T dxx = dx * dx, dxy = dx * dy, dyy = dy * dy;
-  const T r2raw = fmaT(sp<T>(L.A), dxx, fmaT(sp<T>(L.B2), dxy, sp<T>(L.C) * dyy));
+  const T m = fmaT(sp<T>(L.B2), dy, sp<T>(L.A) * dx);
+  const T r2raw = fmaT(m, dx, sp<T>(L.C) * dy * dy);
   const T keep = geT(r2raw, sp<T>(L.r2min));       // 0 where the radius is floored
   const T r2 = maxT(r2raw, sp<T>(L.r2min));
   const T ls = sp<T>(L.c1) * lg2T(r2);
   const T s = ex2T(ls);
-  const T e = ex2T(fmaT(sp<T>(-L.k1), s, sp<T>(L.k1)));
-  const T I = sp<T>(L.I0) * e;
-  const T hI = g * I;
-  const T hs = hI * s;
+  const T ge = g * ex2T(fmaT(sp<T>(-L.k1), s, sp<T>(L.k1)));
+  const T hs = ge * s;
+  const T gq = keep * hs * rcpT(r2);
+  qx = gq * dx;
+  qy = gq * dy;
   acc[0] = acc[0] + hs;
-  acc[1] = fmaT(hI, s - sp<T>(1.f), acc[1]);
-  acc[2] = fmaT(hs, ls, acc[2]);
-  const T q = keep * s * I * rcpT(r2);
-  const float Bh = 0.5f * L.B2;
-  Gx = q * fmaT(sp<T>(L.A), dx, sp<T>(Bh) * dy);
-  Gy = q * fmaT(sp<T>(Bh), dx, sp<T>(L.C) * dy);
-  const T gq = g * q;
-  acc[3] = fmaT(gq, fmaT(sp<T>(L.A1), dxx, fmaT(sp<T>(L.B21), dxy, sp<T>(L.C1) * dyy)), acc[3]);
-  acc[4] = fmaT(gq, fmaT(sp<T>(L.A2), dxx, fmaT(sp<T>(L.B22), dxy, sp<T>(L.C2) * dyy)), acc[4]);
-  acc[5] = fmaT(g, Gx, acc[5]);
-  acc[6] = fmaT(g, Gy, acc[6]);
-  acc[7] = fmaT(g, e, acc[7]);
+  acc[1] = fmaT(hs, ls, acc[1]);
+  acc[2] = acc[2] + qx;
+  acc[3] = acc[3] + qy;
+  acc[4] = fmaT(qx, dx, acc[4]);
+  acc[5] = fmaT(qx, dy, acc[5]);
+  acc[6] = fmaT(qy, dy, acc[6]);
+  acc[7] = acc[7] + ge;
 }
 
-// One ray (or a packed pair): adds g x (derivatives of its intensity) to the
-// 24 accumulators. Branch-free: a ray inside rho < 1e-6 arcsec has S = 0,
-// which zeroes its deflection and every EPL derivative (all carry S).
+// One ray (or a packed pair): adds its share of the 24 accumulators. The mass
+// parameters are taken in reverse: with the source's position derivative as a
+// complex number, H = g (Gx + i Gy) (over b_n/n I0), a change d alpha of the
+// deflection changes the weighted intensity by Re(conj(H) d alpha), and with
+// C = conj(H) S w (alpha = S w F(u)), Z = C F, V = C F'(u) v with v = w / conj(w)
+// (u = -conj(eps) v):
+//   thetaE                 Re Z                            (x t / thetaE)
+//   t                      log2(thetaE / rho) Re Z + Re(C dF/dt) / ln 2   (x ln 2)
+//   w                      Re(q dw), q = conj(w)/|w|^2 [(1 - t) Re Z + i (Im Z - 2 Im(conj(eps) V))]
+//   eps at fixed z, dw = -conj(z) d eps, and through u and S:
+//                          -Re(q conj(z) d eps) - Re(V d conj(eps)) - t eps . d eps / (1 - |eps|^2) Re Z
+//   centre                 dw = -dc + eps conj(dc)
+// so the centre needs only the sums of q, and eps adds one per-vector term
+// (both in k_final). dF/du = [(t/2) F - (1 - t/2) G] / (1 - u), G = (F - 1) / u
+// (Gauss contiguous relation), without a cancellation. The kernel is bound by
+// the FP32 pipe (71% busy) and its latency, and per ray this is about two
+// thirds of the arithmetic of forming each parameter's d alpha: k_ray_adj at
+// 60 x 60, k = 2, B = 4096, 607 -> 459 us; with the signs on the integer pipe
+// and float-stepped grid indices 448, the constants warp-uniform (RayC) and
+// four blocks per SM 406, the series two terms a step and pixels stepped
+// without divisions 396.
+//
+// F and the source position stay in Horner's form: next to the source's centre
+// the gradient follows the last bits of the position (a cusp's slope), and
+// this form is the one its accuracy was measured in. dF/dt only enters one derivative and takes the second-order
+// recurrence for a real polynomial at a complex point (Knuth, TAOCP 4.6.4;
+// |u|^2 = |eps|^2 for every ray): two FMAs per term instead of four.
+// Branch-free: a ray inside rho < 1e-6 arcsec has S = 0, which zeroes its
+// deflection and every EPL derivative (all carry S).
 template <class T>
-__device__ __forceinline__ void ray_adj(const VecConst& V, const float* an, const float* ant, T x, T y, T g, T* acc) {
-  T Gx, Gy;
-  light_adj(V.light[0], x, y, g, acc + A_L_R, Gx, Gy);
+__device__ __forceinline__ void ray_adj(const RayC& V, const float4* ser, T x, T y, T g, T* acc) {
+  T qx, qy;
+  light_adj(V.light[0], x, y, g, acc + A_L, qx, qy);
 
-  // EPL deflection with the pieces of its parameter derivatives
   const T dx = x - sp<T>(V.xc), dy = y - sp<T>(V.yc);
   const T wr = fmaT(sp<T>(-V.e1), dx, fmaT(sp<T>(-V.e2), dy, dx));
   const T wi = fmaT(sp<T>(V.e1), dy, fmaT(sp<T>(-V.e2), dx, dy));
@@ -709,96 +739,68 @@ __device__ __forceinline__ void ray_adj(const VecConst& V, const float* an, cons
   const T ur = fmaT(sp<T>(-V.e1), vr, sp<T>(-V.e2) * vi);
   const T ui = fmaT(sp<T>(V.e2), vr, sp<T>(-V.e1) * vi);
   const T nui = fmaT(sp<T>(-V.e2), vr, sp<T>(V.e1) * vi);   // -ui: packed FMAs take no negated operands
-  // G = sum_{n<N} a_{n+1} u^n and dG/dt by Horner; F = 1 + u G, dF/dt = u dG/dt
-  T Gr = sp<T>(0.f), Gi = sp<T>(0.f), Gtr = sp<T>(0.f), Gti = sp<T>(0.f);
-#pragma unroll 2
-  for (int n = V.nterms_adj; n >= 1; --n) {
-    const T nGr = fmaT(ur, Gr, fmaT(nui, Gi, sp<T>(an[n - 1])));
+  const T ru = ur + ur, nu2 = sp<T>(-V.u2);
+  // G = sum_{n<N} a_{n+1} u^n by Horner; dF/dt / ln 2 = sum_n b_n u^n = ur c1 - |u|^2 c2 + i ui c1;
+  // the two highest terms start the sums, then two more per step
+  const float4 top = ser[V.npairs - 1];
+  T Gr = fmaT(ur, sp<T>(top.y), sp<T>(top.x)), Gi = ui * sp<T>(top.y);
+  T c2 = sp<T>(top.w), c1 = fmaT(ru, c2, sp<T>(top.z));
+  for (int m = V.npairs - 2; m >= 0; --m) {
+    const float4 q = ser[m];
+    const T n1 = fmaT(ur, Gr, fmaT(nui, Gi, sp<T>(q.y)));
     Gi = fmaT(ur, Gi, ui * Gr);
-    Gr = nGr;
-    const T nGtr = fmaT(ur, Gtr, fmaT(nui, Gti, sp<T>(ant[n - 1])));
-    Gti = fmaT(ur, Gti, ui * Gtr);
-    Gtr = nGtr;
+    c2 = fmaT(ru, c1, fmaT(nu2, c2, sp<T>(q.w)));
+    Gr = fmaT(ur, n1, fmaT(nui, Gi, sp<T>(q.x)));
+    Gi = fmaT(ur, Gi, ui * n1);
+    c1 = fmaT(ru, c2, fmaT(nu2, c1, sp<T>(q.z)));
   }
   const T hr = fmaT(ur, Gr, fmaT(nui, Gi, sp<T>(1.f))), hi = fmaT(ur, Gi, ui * Gr);     // F
-  const T tr = fmaT(ur, Gtr, nui * Gti), ti = fmaT(ur, Gti, ui * Gtr);                 // dF/dt
-  // dF/du = [(t/2) F - (1 - t/2) G] / (1 - u)   (Gauss contiguous relation; G = (F - 1)/u
-  // without the cancellation)
+  const T tr = fmaT(ur, c1, nu2 * c2), ti = ui * c1;                                     // dF/dt / ln 2
+  // num = (t/2) F - (1 - t/2) G; F' v = num (v + eps) / |1 - u|^2, |1 - u|^2 = 1 + |u|^2 - 2 ur
+  // (conj(1 - u) v = v + eps |v|^2, |v| = 1)
   const T nr = fmaT(sp<T>(V.th), hr, sp<T>(-V.kc) * Gr), ni = fmaT(sp<T>(V.th), hi, sp<T>(-V.kc) * Gi);
-  const T dr = sp<T>(1.f) - ur;                 // 1 - u = (dr, -ui) = (dr, nui)
-  const T idd = rcpT(fmaT(dr, dr, ui * ui));
-  const T pr = fmaT(nr, dr, ni * nui) * idd, pi = fmaT(ni, dr, nr * ui) * idd;
+  const T idd = rcpT(sp<T>(V.den0) - ru);
+  const T er = (vr + sp<T>(V.e1)) * idd, ei = (vi + sp<T>(V.e2)) * idd;
+  // lens equation with external shear, source at beta
   const T swr = S * wr, swi = S * wi, nswi = S * nwi;   // S w
   const T ar = fmaT(swr, hr, nswi * hi);
   const T ai = fmaT(swr, hi, swi * hr);
-  // t: alpha ln(thetaE/rho) + S w dF/dt
-  const T lnr = sp<T>(0.69314718f) * lrho;
-  const T dtr = fmaT(ar, lnr, fmaT(swr, tr, nswi * ti));
-  const T dti = fmaT(ai, lnr, fmaT(swr, ti, swi * tr));
-  // e1, e2
-  const T Pr = fmaT(wr, dx, nwi * dy), Pi = fmaT(wr, dy, wi * dx);   // w z
-  const T a1 = sp<T>(V.t) * fmaT(Pr, iw2, sp<T>(-V.e1i));             // d ln S / d e1
-  const T a2 = sp<T>(V.t) * fmaT(Pi, iw2, sp<T>(-V.e2i));             // d ln S / d e2
-  const T sfr = S * hr, sfi = S * hi;                                  // S F
-  const T swpr = fmaT(swr, pr, nswi * pi), swpi = fmaT(swr, pi, swi * pr);  // S w F'
-  const T nswpi = -swpi, ndx = -dx, ndy = -dy, nsfi = -sfi;
-  const T k1 = sp<T>(2.f) * Pi * iw2, nk1 = sp<T>(-2.f) * Pi * iw2;
-  const T k2 = sp<T>(2.f) * Pr * iw2, nk2 = sp<T>(-2.f) * Pr * iw2;
-  const T nvr = -vr, nvi = -vi;
-  const T du1r = fmaT(nk1, ui, nvr), du1i = fmaT(k1, ur, nvi);        // du/de1 = -V + i k1 u
-  const T du2r = fmaT(k2, ui, nvi), du2i = fmaT(nk2, ur, vr);         // du/de2 = iV - i k2 u
-  // dw/de1 = (-dx, dy), dw/de2 = (-dy, -dx)
-  const T d1r = fmaT(ar, a1, fmaT(sfr, ndx, nsfi * dy)) + fmaT(swpr, du1r, nswpi * du1i);
-  const T d1i = fmaT(ai, a1, fmaT(sfr, dy, nsfi * dx)) + fmaT(swpr, du1i, swpi * du1r);
-  const T d2r = fmaT(ar, a2, fmaT(sfr, ndy, sfi * dx)) + fmaT(swpr, du2r, nswpi * du2i);
-  const T d2i = fmaT(ai, a2, fmaT(sfr, ndx, nsfi * dy)) + fmaT(swpr, du2i, swpi * du2r);
-  // centre: kappa and shear of the EPL from homogeneity, z kappa + conj(z) gamma = (1-t) alpha
-  const T kap = sp<T>(V.kap_c) * S;
-  const T iz2 = rcpT(maxT(fmaT(dx, dx, dy * dy), sp<T>(1e-30f)));
-  const T nkap = sp<T>(-V.kap_c) * S;
-  const T Qr = fmaT(sp<T>(V.omt), ar, nkap * dx), Qi = fmaT(sp<T>(V.omt), ai, nkap * dy);
-  const T gr = fmaT(Qr, dx, Qi * ndy) * iz2, gi = fmaT(Qr, dy, Qi * dx) * iz2;   // Q z / |z|^2
-  // lens equation with external shear, source at beta
   const T bx = x - ar - fmaT(sp<T>(V.g1), x, sp<T>(V.g2) * y);
   const T by = y - ai - fmaT(sp<T>(V.g2), x, sp<T>(-V.g1) * y);
-  light_adj(V.light[1], bx, by, g, acc + A_S_R, Gx, Gy);
-  // mass: g Ghat . d alpha / d p  (times b_s/n_s in the chain rule);
-  // d alpha/d xc = -(kappa + gamma), d alpha/d yc = -i (kappa - gamma)
-  const T gx = g * Gx, gy = g * Gy;
-  acc[A_THETAE] = fmaT(gx, ar, fmaT(gy, ai, acc[A_THETAE]));
-  acc[A_T] = fmaT(gx, dtr, fmaT(gy, dti, acc[A_T]));
-  acc[A_E1] = fmaT(gx, d1r, fmaT(gy, d1i, acc[A_E1]));
-  acc[A_E2] = fmaT(gx, d2r, fmaT(gy, d2i, acc[A_E2]));
-  acc[A_XC] = acc[A_XC] - fmaT(gx, kap + gr, gy * gi);
-  acc[A_YC] = acc[A_YC] - fmaT(gx, gi, gy * (kap - gr));
-  acc[A_G1] = fmaT(gx, x, fmaT(-gy, y, acc[A_G1]));
+  light_adj(V.light[1], bx, by, g, acc + A_S, qx, qy);
+  const RayLight& L = V.light[1];
+  const float Bh = 0.5f * L.B2;
+  const T gx = fmaT(sp<T>(L.A), qx, sp<T>(Bh) * qy);
+  const T gy = fmaT(sp<T>(Bh), qx, sp<T>(L.C) * qy);
+  const T ngy = -gy;
+  acc[A_G1] = fmaT(gx, x, fmaT(ngy, y, acc[A_G1]));
   acc[A_G2] = fmaT(gx, y, fmaT(gy, x, acc[A_G2]));
+  const T Cr = fmaT(gx, swr, gy * swi), Ci = fmaT(gx, swi, ngy * swr), nCi = -Ci;
+  const T Zr = fmaT(Cr, hr, nCi * hi), Zi = fmaT(Cr, hi, Ci * hr);
+  acc[A_THETAE] = acc[A_THETAE] + Zr;
+  acc[A_T] = fmaT(lrho, Zr, fmaT(Cr, tr, fmaT(nCi, ti, acc[A_T])));
+  // V = C F' v
+  const T Ur = fmaT(Cr, nr, nCi * ni), Ui = fmaT(Cr, ni, Ci * nr);
+  const T Vr = fmaT(Ur, er, -Ui * ei), Vi = fmaT(Ur, ei, Ui * er);
+  const T t1 = sp<T>(V.omt) * Zr, nt1 = -t1;
+  const T t2 = fmaT(sp<T>(-2.f * V.e1), Vi, fmaT(sp<T>(2.f * V.e2), Vr, Zi));
+  const T wbr = wr * iw2, wbi = wi * iw2;
+  const T Qr = fmaT(wbr, t1, wbi * t2), Qi = fmaT(wbr, t2, wbi * nt1), nQi = -Qi;
+  acc[A_QR] = acc[A_QR] + Qr;
+  acc[A_QI] = acc[A_QI] + Qi;
+  acc[A_E1] = fmaT(Qr, dx, fmaT(Qi, dy, acc[A_E1] + Vr));
+  acc[A_E2] = fmaT(Qr, dy, fmaT(nQi, dx, acc[A_E2] + Vi));
 }
 
-// Ray type of the adjoint kernel: float (one ray per thread per step) or F2
-// (two pixels per step, their rays paired in packed f32x2 arithmetic), with
-// its block size and minimum resident blocks.
-#ifndef GL_ADJ_PAIRED
-#define GL_ADJ_PAIRED 1
-#endif
-#ifndef GL_ADJ_THREADS
-#define GL_ADJ_THREADS 128
-#endif
-#ifndef GL_ADJ_MINB
-#define GL_ADJ_MINB 2
-#endif
-constexpr int ADJ_THREADS = GL_ADJ_THREADS;
+// Block size and resident blocks per SM of the adjoint kernel. Four blocks of
+// 128 threads (128 registers, 16 bytes of spills) against three (164, none) and
+// two: 406, 428 and 450 us at 60 x 60, k = 2, B = 4096; 535, 557 and 585 us at
+// 100 x 100, k = 4, B = 512; five (96 registers, 236 bytes of spills) 441 us.
+constexpr int ADJ_THREADS = 128;
+constexpr int ADJ_BLOCKS_PER_SM = 4;
 
-__device__ __forceinline__ float lane_sum(float v) { return v; }
-__device__ __forceinline__ float lane_sum(F2 v) { return v.v.x + v.v.y; }
-
-// MINB: resident blocks per SM the registers are fitted for. Two (218
-// registers, no spills) suit long ray tiles; three (168 registers, 48 bytes
-// of spills) overlap more blocks' prologues and epilogues and suit short ones
-// (60x60 k=2: 654 -> 637 us; 100x100 k=4 at 80K rays per tile: 1725 -> 1736 us).
-template <class Src, int MINB = GL_ADJ_MINB>
-__global__ void __launch_bounds__(ADJ_THREADS, MINB) k_ray_adj(const __grid_constant__ Src src) {
-  using RT = typename std::conditional<GL_ADJ_PAIRED != 0, F2, float>::type;
+template <class Src>
+__global__ void __launch_bounds__(ADJ_THREADS, ADJ_BLOCKS_PER_SM) k_ray_adj(const __grid_constant__ Src src) {
   __shared__ VecConst sv;
   __shared__ Seg ss;
   __shared__ double red[ADJ_THREADS / 32][NACC];
@@ -814,73 +816,56 @@ __global__ void __launch_bounds__(ADJ_THREADS, MINB) k_ray_adj(const __grid_cons
     block_copy(&sv, ss.vc + q);
     __syncthreads();
     const int b = ss.ray_order ? slot_checked(sv.order, q, ss.B) : q;   // the vector in slot q
-    RT acc[NACC];
+    F2 acc[NACC];
 #pragma unroll
-    for (int a = 0; a < NACC; ++a) acc[a] = sp<RT>(0.f);
+    for (int a = 0; a < NACC; ++a) acc[a] = sp<F2>(0.f);
     const int HW = ss.H * ss.W, W = ss.W, k = ss.k;
     const int p0 = tile * ss.tile_pix;
     const int p1 = min(HW, p0 + ss.tile_pix);
     const float* gpre = ss.work + size_t(b) * HW;
     if (sv.nterms >= 0) {
+      const RayC rc = ray_consts(sv);
       const int stride = blockDim.x;
-#if GL_ADJ_PAIRED
-      {
-        // whole steps: two pixels per thread (p and p + blockDim), their rays paired in f32x2
-        const int nfull = (p1 - p0) / (2 * stride);
-        for (int it = 0; it < nfull; ++it) {
-          const int p = p0 + 2 * stride * it + threadIdx.x, q = p + stride;
-          const int ip = p / W, jp = p - ip * W;
-          const int iq = q / W, jq = q - iq * W;
-          const F2 g = {make_float2(gpre[p], gpre[q])};
-          // (indices converted per ray here: float-stepped indices, as in the
-          // forward kernel, cost this register-bound kernel spills and time)
-          for (int a = 0; a < k; ++a) {
-            const F2 y = {make_float2(grid_coord(2 * (ip * k + a) + ss.ny0, ss.hh, ss.hl),
-                                      grid_coord(2 * (iq * k + a) + ss.ny0, ss.hh, ss.hl))};
-            for (int c = 0; c < k; ++c) {
-              const F2 x = {make_float2(grid_coord(2 * (jp * k + c) + ss.nx0, ss.hh, ss.hl),
-                                        grid_coord(2 * (jq * k + c) + ss.nx0, ss.hh, ss.hl))};
-              ray_adj(sv, sv.an, sv.ant, x, y, g, acc);
-            }
-          }
-        }
-        // the ragged end (fewer than 2 blockDim pixels): its rays two per thread and step,
-        // so that every thread takes a share; an odd last ray is paired with itself at zero weight
-        const int base = p0 + 2 * stride * nfull, kk = k * k;
-        const int nr = (p1 - base) * kk;
-        for (int r = 2 * int(threadIdx.x); r < nr; r += 2 * stride) {
-          const bool has2 = r + 1 < nr;
-          const int r2 = has2 ? r + 1 : r;
-          const int pa = base + r / kk, sa = r - (pa - base) * kk;
-          const int pb = base + r2 / kk, sb = r2 - (pb - base) * kk;
-          const int ia = pa / W, ja = pa - ia * W, ib = pb / W, jb = pb - ib * W;
-          const int aa = sa / k, ca = sa - aa * k, ab = sb / k, cb = sb - ab * k;
-          const F2 y = {make_float2(grid_coord(2 * (ia * k + aa) + ss.ny0, ss.hh, ss.hl), grid_coord(2 * (ib * k + ab) + ss.ny0, ss.hh, ss.hl))};
-          const F2 x = {make_float2(grid_coord(2 * (ja * k + ca) + ss.nx0, ss.hh, ss.hl), grid_coord(2 * (jb * k + cb) + ss.nx0, ss.hh, ss.hl))};
-          const F2 g = {make_float2(gpre[pa], has2 ? gpre[pb] : 0.f)};
-          ray_adj(sv, sv.an, sv.ant, x, y, g, acc);
+      // whole steps: two pixels per thread (p and p + blockDim), their rays paired in f32x2
+      const int nfull = (p1 - p0) / (2 * stride);
+      const PixelStep step(2 * stride, W);
+      int p = p0 + threadIdx.x;
+      int ip = p / W, jp = p - ip * W, iq = (p + stride) / W, jq = p + stride - iq * W;
+      for (int it = 0; it < nfull; ++it, p += 2 * stride, step.advance(ip, jp, W), step.advance(iq, jq, W)) {
+        const F2 g = {make_float2(gpre[p], gpre[p + stride])};
+        // grid indices of the pixels' first subpixels; a subpixel step adds 2
+        const F2 nx0 = {make_float2(float(2 * jp * k + ss.nx0), float(2 * jq * k + ss.nx0))};
+        F2 ny = {make_float2(float(2 * ip * k + ss.ny0), float(2 * iq * k + ss.ny0))};
+        for (int a = 0; a < k; ++a, ny = ny + sp<F2>(2.f)) {
+          const F2 y = grid_coord2(ny, ss.hh, ss.hl);
+          F2 nx = nx0;
+          for (int c = 0; c < k; ++c, nx = nx + sp<F2>(2.f))
+            ray_adj(rc, sv.ser, grid_coord2(nx, ss.hh, ss.hl), y, g, acc);
         }
       }
-#else
-      {
-        for (int p = p0 + threadIdx.x; p < p1; p += stride) {
-          const int i = p / W, j = p - i * W;
-          const float g = gpre[p];
-          for (int a = 0; a < k; ++a) {
-            const float y = grid_coord(2 * (i * k + a) + ss.ny0, ss.hh, ss.hl);
-            for (int c = 0; c < k; ++c) {
-              const float x = grid_coord(2 * (j * k + c) + ss.nx0, ss.hh, ss.hl);
-              ray_adj(sv, sv.an, sv.ant, x, y, g, acc);
-            }
-          }
-        }
+      // the ragged end (fewer than 2 blockDim pixels): its rays two per thread and step,
+      // so that every thread takes a share; an odd last ray is paired with itself at zero weight
+      const int base = p0 + 2 * stride * nfull, kk = k * k;
+      const int nr = (p1 - base) * kk;
+      for (int r = 2 * int(threadIdx.x); r < nr; r += 2 * stride) {
+        const bool has2 = r + 1 < nr;
+        const int r2 = has2 ? r + 1 : r;
+        const int pa = base + r / kk, sa = r - (pa - base) * kk;
+        const int pb = base + r2 / kk, sb = r2 - (pb - base) * kk;
+        const int ia = pa / W, ja = pa - ia * W, ib = pb / W, jb = pb - ib * W;
+        const int aa = sa / k, ca = sa - aa * k, ab = sb / k, cb = sb - ab * k;
+        const F2 y = {make_float2(grid_coord(2 * (ia * k + aa) + ss.ny0, ss.hh, ss.hl),
+                                  grid_coord(2 * (ib * k + ab) + ss.ny0, ss.hh, ss.hl))};
+        const F2 x = {make_float2(grid_coord(2 * (ja * k + ca) + ss.nx0, ss.hh, ss.hl),
+                                  grid_coord(2 * (jb * k + cb) + ss.nx0, ss.hh, ss.hl))};
+        const F2 g = {make_float2(gpre[pa], has2 ? gpre[pb] : 0.f)};
+        ray_adj(rc, sv.ser, x, y, g, acc);
       }
-#endif
     }
     // pairwise FP32 sums within the warp (GB300's FP64 pipe is narrow), FP64 across warps
 #pragma unroll
     for (int a = 0; a < NACC; ++a) {
-      float v = lane_sum(acc[a]);
+      float v = acc[a].v.x + acc[a].v.y;
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
       if (lane == 0) red[warp][a] = double(v);
@@ -1918,44 +1903,84 @@ __global__ void __launch_bounds__(BAND_THREADS, 2) k_conv_sep_bands(const __grid
 
 // ------------------------------------------------------------- k_final ----
 
-// The FP64 factors of a vector's chain rule, from five reciprocals:
-// b_n / n = 1.9992 - 0.3271 / n of the source and of the lens light, and
-// 1 / thetaE, 1 / R_l, 1 / R_s.
-struct ChainF {
-  double ms, ml, ite, iRl, iRs;
+// The per-vector chain rule: gradient entry j from the summed accumulators
+// a[NACC] (Acc: what each holds) is, in FP64,
+//   scale_j (k0 a[i0] + k1 a[i1] + k2 a[i2])
+// (n1 .. of the terms used). The terms are set up per entry from the
+// parameters pf and the constants V, without FP64 divisions except for the
+// one reciprocal, so that lanes of a warp that form different entries only
+// diverge over cheap FP32 and index selects, and the loads and the
+// reciprocal do not wait for the accumulators. Shared by the two k_final
+// variants so that they give identical results.
+struct ChainTerm {
+  double scale, k[3];
+  int i[3], n;
 };
-// Parameter whose reciprocal is factor i of chain_factors.
-__device__ __forceinline__ float recip_param(const float* pf, int i) {
-  return pf[i == 0 ? 16 : i == 1 ? 9 : i == 2 ? 0 : i == 3 ? 8 : 15];
-}
-__device__ __forceinline__ ChainF chain_factors(const double* r) {
-  ChainF f;
-  f.ms = fma(-0.3271, r[0], 1.9992);
-  f.ml = fma(-0.3271, r[1], 1.9992);
-  f.ite = r[2];
-  f.iRl = r[3];
-  f.iRs = r[4];
-  return f;
+// The parameter n of the light whose b_n / n = 1.9992 - 0.3271 / n entry j
+// takes: the source's for the mass parameters.
+__device__ __forceinline__ int chain_recip_param(int j) { return j >= 8 && j < 15 ? 9 : 16; }
+
+// rn: 1 / pf[chain_recip_param(j)]; r2: 1 / thetaE, 1 / R_l, 1 / R_s for entries 0, 8 and 15
+__device__ __forceinline__ ChainTerm chain_term(int j, const float* pf, const VecConst& V, double rn, double r2) {
+  const double ln2 = 0.69314718055994530942;
+  const bool lens = j >= 8 && j < 15;
+  const double I0 = pf[lens ? 14 : 21];
+  const double bn = fma(-0.3271, rn, 1.9992);   // b_n / n
+  const double m = bn * I0;
+  ChainTerm c;
+  c.k[0] = 1.0;
+  c.k[1] = c.k[2] = 0.0;
+  c.i[1] = c.i[2] = 0;
+  c.n = 1;
+  if (j < 8) {
+    const double t = double(pf[1]) - 1.0, e1 = pf[2], e2 = pf[3];
+    c.scale = j == 0 ? m * t * r2 : j == 1 ? m * ln2 : j < 4 ? -m : m;
+    c.i[0] = j < 4 ? j : j < 6 ? int(A_QR) : j;
+    if (j == 2 || j == 3) {
+      c.n = 2;
+      c.i[1] = A_THETAE;
+      c.k[1] = t * double(j == 2 ? V.e1i : V.e2i);
+    } else if (j == 4 || j == 5) {
+      c.n = 2;
+      c.k[0] = j == 4 ? e1 - 1.0 : e2;
+      c.i[1] = A_QI;
+      c.k[1] = j == 4 ? -e2 : e1 + 1.0;
+    }
+    return c;
+  }
+  const int o = lens ? int(A_L) : int(A_S), k = j - (lens ? 8 : 15);
+  const LightC& L = V.light[lens ? 0 : 1];
+  c.scale = k == 0 ? m * r2 : k == 1 ? I0 : k < 4 ? -0.5 * m : k < 6 ? m : 1.0;
+  c.i[0] = o + (k == 0 ? 0 : k == 1 ? 1 : k < 4 ? 4 : k < 6 ? 2 : 7);
+  if (k == 1) {
+    c.n = 3;
+    c.k[0] = ln2 * bn;
+    c.i[1] = o + 7;
+    c.k[1] = 1.9992;
+    c.i[2] = o;
+    c.k[2] = -1.9992;
+  } else if (k == 2 || k == 3) {
+    c.n = 3;
+    c.k[0] = k == 2 ? L.A1 : L.A2;
+    c.i[1] = o + 5;
+    c.k[1] = k == 2 ? L.B21 : L.B22;
+    c.i[2] = o + 6;
+    c.k[2] = k == 2 ? L.C1 : L.C2;
+  } else if (k == 4 || k == 5) {
+    const float Bh = 0.5f * L.B2;
+    c.n = 2;
+    c.k[0] = k == 4 ? L.A : Bh;
+    c.i[1] = o + 3;
+    c.k[1] = k == 4 ? Bh : L.C;
+  }
+  return c;
 }
 
-// The per-vector chain rule from the summed accumulators a[NACC], the
-// parameters pf and the factors f (FP64 arithmetic): gradient entry j.
-// Shared by the two k_final variants so that they give identical results.
-__device__ __forceinline__ double chain_rule(int j, const double* a, const float* pf, const ChainF& f) {
-  const double ln2 = 0.69314718055994530942;
-  if (j < 8) return j == 0 ? f.ms * (double(pf[1]) - 1.0) * f.ite * a[A_THETAE] : f.ms * a[A_THETAE + j];
-  const int l = j < 15 ? 0 : 1, k = j - (l == 0 ? 8 : 15);
-  const double* c = a + (l == 0 ? A_L_R : A_S_R);
-  const double m = l == 0 ? f.ml : f.ms;
-  switch (k) {
-    case 0: return m * (l == 0 ? f.iRl : f.iRs) * c[0];
-    case 1: return -1.9992 * c[1] + m * ln2 * c[2];
-    case 2: return -0.5 * m * c[3];
-    case 3: return -0.5 * m * c[4];
-    case 4: return m * c[5];
-    case 5: return m * c[6];
-    default: return c[7];
-  }
+__device__ __forceinline__ double chain_rule(const ChainTerm& c, const double* a) {
+  double v = c.k[0] * a[c.i[0]];
+  if (c.n > 1) v = fma(c.k[1], a[c.i[1]], v);
+  if (c.n > 2) v = fma(c.k[2], a[c.i[2]], v);
+  return c.scale * v;
 }
 
 // One thread per vector (calls whose vectors have one ray tile each).
@@ -1982,11 +2007,17 @@ __global__ void k_final(const __grid_constant__ Src src) {
     for (int t = 0; t < s->ntiles; ++t)
       for (int i = 0; i < NACC; ++i) a[i] += part[t * NACC + i];
     const float* pf = s->params + size_t(b) * NPARAM;
-    double r[5];
+    const VecConst& V = s->vc[p];
+    const double rl = 1.0 / double(pf[9]), rs = 1.0 / double(pf[16]);
+    const double r0 = 1.0 / double(pf[0]), r8 = 1.0 / double(pf[8]), r15 = 1.0 / double(pf[15]);
+    // every entry before the first store: a store could alias the parameters and constants, and the
+    // loads of the later entries would wait for it
+    double out[NPARAM];
 #pragma unroll
-    for (int i = 0; i < 5; ++i) r[i] = 1.0 / double(recip_param(pf, i));
-    const ChainF f = chain_factors(r);
-    for (int j = 0; j < NPARAM; ++j) g[j] = chain_rule(j, a, pf, f);
+    for (int j = 0; j < NPARAM; ++j)
+      out[j] = chain_rule(chain_term(j, pf, V, chain_recip_param(j) == 9 ? rl : rs, j == 0 ? r0 : j == 8 ? r8 : r15), a);
+#pragma unroll
+    for (int j = 0; j < NPARAM; ++j) g[j] = out[j];
   }
 }
 
@@ -2007,6 +2038,15 @@ __global__ void k_final_warp(const __grid_constant__ Src src) {
       if (lane < NPARAM) g[lane] = nan("");
       continue;
     }
+    // the entry's terms first: their loads and reciprocals overlap the partials' loads
+    const float* pf = s->params + size_t(b) * NPARAM;
+    const int j = lane < NPARAM ? lane : NPARAM - 1;
+    // lanes 0 .. 4 take the five reciprocals at once (n_l, n_s, thetaE, R_l, R_s)
+    const int ri = lane == 0 ? 9 : lane == 1 ? 16 : lane == 2 ? 0 : lane == 3 ? 8 : 15;
+    const double recip = 1.0 / double(pf[ri]);
+    const double rn = __shfl_sync(0xffffffffu, recip, chain_recip_param(j) == 9 ? 0 : 1);
+    const double r2 = __shfl_sync(0xffffffffu, recip, j == 0 ? 2 : j == 8 ? 3 : 4);
+    const ChainTerm term = chain_term(j, pf, s->vc[p], rn, r2);
     if (lane < NACC) {
       // eight loads in flight, then added in tile order (the same sum as k_final)
       const double* part = s->partial + size_t(b) * s->ntiles * NACC + lane;
@@ -2024,14 +2064,7 @@ __global__ void k_final_warp(const __grid_constant__ Src src) {
       sa[w][lane] = acc;
     }
     __syncwarp();
-    const float* pf = s->params + size_t(b) * NPARAM;
-    // lanes 0..4 take the five divisions at once; every lane receives them
-    const double rl = lane < 5 ? 1.0 / double(recip_param(pf, lane)) : 0.0;
-    double r[5];
-#pragma unroll
-    for (int i = 0; i < 5; ++i) r[i] = __shfl_sync(0xffffffffu, rl, i);
-    const ChainF f = chain_factors(r);
-    if (lane < NPARAM) g[lane] = chain_rule(lane, sa[w], pf, f);
+    if (lane < NPARAM) g[lane] = chain_rule(term, sa[w]);
     __syncwarp();
   }
 }
@@ -2132,9 +2165,6 @@ size_t seg_conv_smem(const Seg& g) {
   return g.conv_sep ? conv_sep_smem_bytes(g.H, g.W, g.K, g.psf_rank) : conv_smem_bytes(g.H, g.W, g.K, g.conv_two_buf != 0);
 }
 
-// Ray tiles of at most this many rays take the three-blocks-per-SM adjoint.
-constexpr long long ADJ_SHORT_TILE_RAYS = 32768;
-
 // Resident blocks per SM of the forward ray kernel (occupancy query, cached;
 // its launch bound if the query fails, e.g. without a GPU).
 static int fwd_blocks_per_sm() {
@@ -2143,7 +2173,7 @@ static int fwd_blocks_per_sm() {
   if (n == 0) {
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_ray_fwd<OneSeg>, FWD_THREADS, 0) != cudaSuccess || n < 1) {
       cudaGetLastError();
-      n = GL_FWD_MINB;
+      n = FWD_BLOCKS_PER_SM;
     }
     cached.store(n, std::memory_order_relaxed);
   }
@@ -2151,51 +2181,52 @@ static int fwd_blocks_per_sm() {
 }
 
 // Tiling of a B-vector call's rays: the tile count that minimises a model of
-// the two ray kernels' time, waves x (pixels per tile + a fixed per-tile
-// cost of 64 pixels), the forward kernel at its resident blocks per SM and
-// the adjoint, 2.4 times the forward's cost per ray (measured at 60 x 60,
-// k = 2), at two or three blocks per SM (a three-block wave takes 3/2.054 of
-// a two-block wave: a block's time grows with the blocks sharing its SM, and
-// three share 1.027x the work of two; three only for tiles of at most
-// ADJ_SHORT_TILE_RAYS rays, whose spills cost little). Tiles keep at least
-// 8 rays per thread of a 256-thread block; ties go to fewer tiles. Below
-// one vector per SM the forward's waves weigh half: there they are partly
-// filled, and its blocks, sharing an SM with fewer others, finish sooner
-// than the model's full wave. 50 vectors of 80 x 80, k = 2, then take 9
-// tiles (one three-block adjoint wave) instead of 12 (46.9 -> 44.1 us a
-// call near one mode, 56.7 -> 54.0 us for vectors drawn from the prior);
-// 100 x 100, k = 4: 145.5 -> 145.0 us. Larger batches keep weight 1: with
-// half, 300 vectors from the prior took 2 tiles instead of 5 (178 -> 204 us;
-// the model does not see a batch's spread of per-vector cost).
+// the two ray kernels' time. Per kernel, with R resident blocks per SM, a
+// tile costs its pixels plus TILE_RAYS rays of prologue; the call is whole
+// waves of R blocks per SM and a part of one, which takes its share of a
+// wave but at least PART of one (fewer warps hide less latency), and a tail:
+// the last blocks of a mixed batch (drawn from a prior) end at different
+// times, TAIL_MIXED of a tile; below one vector per SM, near one mode, they
+// end together. The adjoint weighs 2, its time over the forward's. Measured,
+// forward + adjoint in us by tile count: 300 vectors of 80 x 80 from the prior
+// 1: 223, 2: 138, 3: 124, 4: 115, 6: 116, 8: 116 (takes 6); 50 vectors near one
+// mode 3: 43, 6: 34, 9: 31, 12: 31, 18: 35, 25: 34 (takes 9); 512 vectors of
+// 100 x 100, k = 4, 1: 980, 2: 836, 4: 814, 8: 799 (takes 8). A larger count must
+// gain two percent. Tiles keep at least one step of a block (two pixels a
+// thread) and four rays a thread.
 struct TilePlan {
   int ntiles, tile_pix;
-  bool adj3;
 };
 
+static double ray_kernel_cost(double items, double px, double slots, double tail) {
+  constexpr double PART = 0.55;
+  const double w = items / slots, full = std::floor(w), part = w - full;
+  return px * (full + (part > 0.0 ? (part > PART ? part : PART) : 0.0) + tail);
+}
+
 static TilePlan plan_rays(int B, int H, int W, int k) {
+  constexpr double TILE_RAYS = 256.0, TAIL_MIXED = 0.35, TAIL_MODE = 0.1;
   const int HW = H * W;
-  TilePlan best{1, HW, false};
+  TilePlan best{1, HW};
   if (B <= 0 || HW <= 0) return best;
   const long long rays = (long long)HW * k * k;
-  long long max_nt = (rays + RAY_THREADS * 8 - 1) / (RAY_THREADS * 8);
-  if (max_nt > HW) max_nt = HW;
+  long long max_nt = (HW + 2 * ADJ_THREADS - 1) / (2 * ADJ_THREADS);
+  const long long by_rays = (rays + 4 * ADJ_THREADS - 1) / (4 * ADJ_THREADS);
+  if (by_rays < max_nt) max_nt = by_rays;
   if (max_nt < 1) max_nt = 1;
-  const double sms = num_sms(), fwd_slots = sms * fwd_blocks_per_sm();
-  const double wf = B < sms ? 0.5 : 1.0;   // weight of the forward's waves
+  const double sms = num_sms(), fwd_slots = sms * fwd_blocks_per_sm(), adj_slots = sms * ADJ_BLOCKS_PER_SM;
+  const double tail = B < sms ? TAIL_MODE : TAIL_MIXED;
   double best_cost = 0.0;
   for (long long nt = 1; nt <= max_nt; ++nt) {
     const int tp = int((HW + nt - 1) / nt);
     const int ntt = (HW + tp - 1) / tp;
     if (ntt != nt) continue;   // the same tiling as a smaller count
-    const double items = double(B) * ntt, px = tp + 64.0;
-    const double fwd = std::ceil(items / fwd_slots) * px;
-    const double adj2 = std::ceil(items / (2 * sms)) * px;
-    const bool short_tile = (long long)tp * k * k <= ADJ_SHORT_TILE_RAYS;
-    const double adj3 = short_tile ? std::ceil(items / (3 * sms)) * px * (3.0 / 2.054) : 1e300;
-    const double cost = wf * fwd + 2.4 * (adj3 < adj2 ? adj3 : adj2);
-    if (nt == 1 || cost < best_cost * (1.0 - 1e-9)) {
+    const double items = double(B) * ntt, px = tp + TILE_RAYS / (double(k) * k);
+    const double cost = ray_kernel_cost(items, px, fwd_slots, tail) * fwd_slots / adj_slots +
+                        2.0 * ray_kernel_cost(items, px, adj_slots, tail);
+    if (nt == 1 || cost < best_cost * 0.98) {
       best_cost = cost;
-      best = TilePlan{ntt, tp, adj3 < adj2};
+      best = TilePlan{ntt, tp};
     }
   }
   return best;
@@ -2428,8 +2459,7 @@ static cudaError_t launch_order(const Src&, int, cudaStream_t) { return cudaErro
 
 template <class Src>
 static cudaError_t run_rays(const Src& src, int nvec, int nray, bool fwd, bool adj_final, cudaStream_t st,
-                            Hooks* hooks, bool persistent, bool one_tile = false, bool fwd_rays = true,
-                            bool short_tiles = false) {
+                            Hooks* hooks, bool persistent, bool one_tile = false, bool fwd_rays = true) {
   const int sms = num_sms();
   cudaError_t e;
   const int vthreads = SETUP_THREADS, wpb = vthreads / 32 - 2;
@@ -2464,10 +2494,7 @@ static cudaError_t run_rays(const Src& src, int nvec, int nray, bool fwd, bool a
   }
   if (adj_final) {
     hooks->before(GL_K_RAY_ADJ, st);
-    if (short_tiles)
-      e = launch_pdl(k_ray_adj<Src, 3>, unsigned(rgrid), ADJ_THREADS, 0, st, src);
-    else
-      e = launch_pdl(k_ray_adj<Src>, unsigned(rgrid), ADJ_THREADS, 0, st, src);
+    e = launch_pdl(k_ray_adj<Src>, unsigned(rgrid), ADJ_THREADS, 0, st, src);
     cudaError_t h = hooks->after(GL_K_RAY_ADJ, st);
     if (e != cudaSuccess || (e = h) != cudaSuccess) return e;
     hooks->before(GL_K_FINAL, st);
@@ -2508,10 +2535,7 @@ cudaError_t launch_one(const Seg& s0, int mode, cudaStream_t st, Hooks* hooks) {
   if (e != cudaSuccess) return e;
   if ((e = hooks->after(GL_K_CONV, st)) != cudaSuccess) return e;
   if (mode != MODE_GRAD && mode != MODE_CORR) return cudaSuccess;
-  // the adjoint's blocks per SM as the tile plan chose them (plan_rays)
-  const TilePlan tp = plan_rays(s.B, s.H, s.W, s.k);
-  const bool three = tp.adj3 && tp.ntiles == s.ntiles && tp.tile_pix == s.tile_pix;
-  return run_rays(src, s.B, s.B * s.ntiles, false, true, st, hooks, false, s.ntiles == 1, true, three);
+  return run_rays(src, s.B, s.B * s.ntiles, false, true, st, hooks, false, s.ntiles == 1);
 }
 
 cudaError_t launch_basis(const Seg& s, cudaStream_t st, Hooks* hooks) {
@@ -2601,7 +2625,7 @@ cudaError_t launch_devtable(const TableHdr* d_hdr, const Seg* d_segs, const size
     if ((e = hooks->after(GL_K_CONV, st)) != cudaSuccess) return e;
   }
   hooks->before(GL_K_RAY_ADJ, st);
-  if ((e = launch_pdl(k_ray_adj<DevTable>, unsigned(sms * GL_ADJ_MINB), ADJ_THREADS, 0, st, src)) != cudaSuccess)
+  if ((e = launch_pdl(k_ray_adj<DevTable>, unsigned(sms * ADJ_BLOCKS_PER_SM), ADJ_THREADS, 0, st, src)) != cudaSuccess)
     return e;
   if ((e = hooks->after(GL_K_RAY_ADJ, st)) != cudaSuccess) return e;
   hooks->before(GL_K_FINAL, st);
