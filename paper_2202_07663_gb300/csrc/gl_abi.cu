@@ -27,6 +27,7 @@ struct gl_system {
   float* d_psf = nullptr;
   // the PSF as psf_rank separable terms (0: convolve with the K x K PSF directly)
   int psf_rank = 0;
+  bool psf_mirror = false;      // the PSF's rows are the same from the top and from the bottom
   float* d_psf_sep = nullptr;   // [psf_rank][2][K]: sigma_r u_r (rows), v_r (columns)
   // scratch, grown on demand
   long long cap_B = 0;
@@ -247,7 +248,7 @@ void partial_need(const gl_system* s, int B, int* ntiles, int* tile_pix, long lo
   *partial = (long long)B * (*ntiles) * gl::NACC;
 }
 
-Seg make_seg(const gl_system* s, const float* params, int B) {
+Seg make_seg(const gl_system* s, const float* params, int B, int ntiles, int tile_pix) {
   Seg g;
   std::memset(&g, 0, sizeof(g));
   g.image = s->d_image;
@@ -268,10 +269,13 @@ Seg make_seg(const gl_system* s, const float* params, int B) {
   g.inv_gain = s->gain_exposure > 0.0 ? float(1.0 / s->gain_exposure) : 0.f;
   g.params = params;
   g.B = B;
-  gl::plan_tiles(B, s->H, s->W, s->k, &g.ntiles, &g.tile_pix);
+  g.ntiles = ntiles;
+  g.tile_pix = tile_pix;
   g.vc = s->d_vc;
   g.work = s->d_work;
   g.partial = s->d_partial;
+  g.psf_mirror = s->psf_mirror ? 1 : 0;
+  g.conv_rows = gl::conv_rows_fit(s->H, s->W, s->K) ? 1 : 0;
   g.conv_two_buf = gl::conv_two_buf(s->H, s->W, s->K) ? 1 : 0;
   g.conv_sep = gl::conv_sep_ok(s->H, s->W, s->K, s->psf_rank) ? 1 : 0;
   return g;
@@ -304,7 +308,7 @@ int run_one(gl_system* s, const float* params, int B, double* ll, double* c2, do
   partial_need(s, B, &ntiles, &tile_pix, &partial);
   int rc = ensure_scratch(s, B, partial);
   if (rc != GL_OK) return rc;
-  Seg g = make_seg(s, params, B);
+  Seg g = make_seg(s, params, B, ntiles, tile_pix);
   g.loglik = ll;
   g.chi2 = c2;
   g.grad = grad;
@@ -328,7 +332,9 @@ size_t scratch_held(const gl_system* s) {
 
 // Segment of a call on sys with every scratch pointer left null.
 gl::Seg seg_without_scratch(const gl_system* s, const float* params, int B) {
-  Seg g = make_seg(s, params, B);
+  int ntiles, tile_pix;
+  gl::plan_tiles(B, s->H, s->W, s->k, &ntiles, &tile_pix);
+  Seg g = make_seg(s, params, B, ntiles, tile_pix);
   g.vc = nullptr;
   g.work = nullptr;
   g.partial = nullptr;
@@ -384,6 +390,9 @@ int create_impl(gl_system** out, const float* image, const std::vector<float>& s
     gl_system_destroy(s);
     return cuda_fail(e, "gl_system_create upload");
   }
+  s->psf_mirror = true;
+  for (int a = 0; a < K / 2; ++a)
+    for (int i = 0; i < K; ++i) s->psf_mirror = s->psf_mirror && psf_area[size_t(a) * K + i] == psf_area[size_t(K - 1 - a) * K + i];
   std::vector<float> fac;
   const int R = psf_separable(psf_area, K, fac);
   if (R > 0 && gl::conv_sep_any(H, W, K, R)) {   // factors kept only where the 1-D passes run
@@ -600,7 +609,7 @@ int gl_loglik_grad_profiled(gl_system* s, const float* params, int B, double* lo
   partial_need(s, B, &ntiles, &tile_pix, &partial);
   rc = ensure_scratch(s, 2LL * B, partial);
   if (rc != GL_OK) return rc;
-  Seg g = make_seg(s, params, B);
+  Seg g = make_seg(s, params, B, ntiles, tile_pix);
   g.sim = s->d_pimg;
   cudaError_t e = gl::launch_basis(g, st, &g_prof);
   if (e != cudaSuccess) return cuda_fail(e, "basis images");
@@ -678,7 +687,7 @@ int gl_loglik_grad_grouped(gl_system* const* systems, const float* const* params
     partial_need(s, B[i], &ntiles, &tile_pix, &partial);
     rc = ensure_scratch(s, B[i], partial);
     if (rc != GL_OK) return rc;
-    Seg sg = make_seg(s, params[i], B[i]);
+    Seg sg = make_seg(s, params[i], B[i], ntiles, tile_pix);
     sg.loglik = loglik_out[i];
     sg.chi2 = chi2_out ? chi2_out[i] : nullptr;
     sg.grad = g ? grad_out[i] : nullptr;

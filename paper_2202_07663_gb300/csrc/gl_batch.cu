@@ -105,6 +105,8 @@ int gl_batcher_create(gl_batcher** out, int max_segments, size_t arena_bytes, in
     if (c < 2 && K > max_K) continue;
     size_t one = gl::conv_smem_bytes(max_H, max_W, K, false), two = gl::conv_smem_bytes(max_H, max_W, K, true);
     size_t sm = gl::conv_two_buf(max_H, max_W, K) ? two : one;
+    // room for the rank-1 separable form of the largest image, where it has one
+    if (c == 2 && gl::conv_sep_ok(max_H, max_W, K, 1)) sm = std::max(sm, gl::conv_sep_smem_bytes(max_H, max_W, K, 1));
     b->conv_smem[c] = sm;
     if (one + 2048 > size_t(optin)) {
       gl_batcher_destroy(b);
@@ -179,6 +181,8 @@ int gl_batcher_run(gl_batcher* b, gl_system* const* systems, const float* const*
     const int c = gl::conv_class(g.K);
     if (g.conv_sep && gl::seg_conv_smem(g) > b->conv_smem[c]) g.conv_sep = 0;
     if (g.conv_two_buf && gl::conv_smem_bytes(g.H, g.W, g.K, true) > b->conv_smem[c]) g.conv_two_buf = 0;
+    if (c == 2 && !g.conv_sep && g.conv_rows && gl::seg_conv_smem(g) > b->conv_smem[c])
+      g.conv_rows = g.conv_two_buf = 0;   // column strips: their rows are narrower
     if (gl::seg_conv_smem(g) > b->conv_smem[c])
       return gl_internal::set_error(GL_ERR_UNSUPPORTED, "segment convolution does not fit the captured shared memory");
     const size_t need = segment_scratch(g);
@@ -209,6 +213,7 @@ int gl_batcher_run(gl_batcher* b, gl_system* const* systems, const float* const*
     gl::Seg g;
     for (int c = 0; c < gl::N_CONV_CLASSES; ++c)
       if (!by_class[c].empty()) g = by_class[c][0];
+    g.conv_rows = gl::conv_rows_fit(g.H, g.W, g.K) ? 1 : 0;
     g.conv_two_buf = gl::conv_two_buf(g.H, g.W, g.K) ? 1 : 0;
     g.conv_sep = gl::conv_sep_ok(g.H, g.W, g.K, g.psf_rank) ? 1 : 0;
     if (b->ran && st != b->last_stream && (e = cudaStreamWaitEvent(st, b->done, 0)) != cudaSuccess)

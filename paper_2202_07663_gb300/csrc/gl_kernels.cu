@@ -883,31 +883,7 @@ __global__ void __launch_bounds__(ADJ_THREADS, ADJ_BLOCKS_PER_SM) k_ray_adj(cons
 // -------------------------------------------------------------- k_conv ----
 
 // out(i, j) = sum_{a,b} ker[a K + b] in[(i + a) Wp + j + b] for the R rows
-// i = i0 .. i0 + R - 1 of column j. The kernel column sits in registers and
-// every input value is read once per kernel column.
-template <int K, int R>
-__device__ __forceinline__ void corr_strip(const float* in, int Wp, const float* ker, int i0, int j, float* acc) {
-#pragma unroll
-  for (int r = 0; r < R; ++r) acc[r] = 0.f;
-  const float* base = in + i0 * Wp + j;
-#pragma unroll 1
-  for (int b = 0; b < K; ++b) {
-    float kc[K];
-#pragma unroll
-    for (int a = 0; a < K; ++a) kc[a] = ker[a * K + b];
-    const float* col = base + b;
-#pragma unroll
-    for (int ii = 0; ii < R + K - 1; ++ii) {
-      const float v = col[ii * Wp];
-#pragma unroll
-      for (int r = 0; r < R; ++r) {
-        const int a = ii - r;
-        if (a >= 0 && a < K) acc[r] = fmaf(kc[a], v, acc[r]);
-      }
-    }
-  }
-}
-
+// i = i0 .. i0 + R - 1 of column j.
 template <int R>
 __device__ __forceinline__ void corr_strip_any(const float* in, int Wp, const float* ker, int K, int i0, int j,
                                                float* acc) {
@@ -946,14 +922,16 @@ __device__ __forceinline__ float warp_sum_f(float v) {
   return v;
 }
 
-// One vector. Shared memory: PSF flipped (convolution) and as given
-// (correlation), the zero-padded binned image and, when it fits
-// (s.conv_two_buf), a second zero-padded buffer for the pixel adjoint;
-// otherwise the adjoint goes through this vector's global work slot.
-// K > 0: compile-time PSF side; K == 0: any odd side (s.K).
-template <int K, int R>
+// One vector by column strips, for images that fit a block's shared memory
+// only without the row strips' pitch (conv_rows_fit). Shared memory: PSF
+// flipped (convolution) and as given (correlation), the zero-padded binned
+// image and, when it fits (s.conv_two_buf), a second zero-padded buffer for
+// the pixel adjoint; otherwise the adjoint goes through this vector's global
+// work slot.
+constexpr int STRIP_ROWS = 8;
 __device__ void conv_vector(const Seg& s, int b, int mode, float* smem, double* red2) {
-  const int Kk = K > 0 ? K : s.K;
+  constexpr int R = STRIP_ROWS;
+  const int Kk = s.K;
   const int H = s.H, W = s.W, HW = H * W;
   const int nstrip = (H + R - 1) / R;
   const int Hp = nstrip * R + Kk - 1, Wp = W + Kk - 1;
@@ -992,8 +970,7 @@ __device__ void conv_vector(const Seg& s, int b, int mode, float* smem, double* 
     const int strip = u / Wr, j = u - strip * Wr;
     if (j >= W) continue;
     const int i0 = strip * R;
-    if (K > 0) corr_strip<(K > 0 ? K : 1), R>(img, Wp, kerF, i0, j, acc);
-    else corr_strip_any<R>(img, Wp, kerF, Kk, i0, j, acc);
+    corr_strip_any<R>(img, Wp, kerF, Kk, i0, j, acc);
 #pragma unroll
     for (int r = 0; r < R; ++r) {
       const int i = i0 + r;
@@ -1060,8 +1037,7 @@ __device__ void conv_vector(const Seg& s, int b, int mode, float* smem, double* 
     const int strip = u / Wr, j = u - strip * Wr;
     if (j >= W) continue;
     const int i0 = strip * R;
-    if (K > 0) corr_strip<(K > 0 ? K : 1), R>(gsrc, Wp, kerU, i0, j, acc);
-    else corr_strip_any<R>(gsrc, Wp, kerU, Kk, i0, j, acc);
+    corr_strip_any<R>(gsrc, Wp, kerU, Kk, i0, j, acc);
 #pragma unroll
     for (int r = 0; r < R; ++r) {
       const int i = i0 + r;
@@ -1087,50 +1063,113 @@ __device__ __forceinline__ float pixel_terms(const Seg& s, int p, float M, float
   return fmaf(0.5f * s.inv_gain, fmaf(t2, iv, -iv), res * iv);
 }
 
-// ---- row-strip convolution for the compile-time PSF sides (11, 21) ----
+// ---- row-strip convolution ----
 //
 // Each thread computes S = 16 consecutive outputs of one image row; the lanes
 // of a warp take consecutive rows. Per kernel row a thread loads the input
 // span (S + K - 1 values) and the kernel row as float4 and does S*K FMAs from
 // registers. The row pitch P (floats) is a multiple of 4 with an odd number
 // of float4 per row, so the 8 lanes of each 128-bit shared-memory phase hit
-// 8 distinct bank groups.
+// 8 distinct bank groups. The sides 11 and 21 are compiled whole; any other
+// odd side runs in groups of 16 taps and one of K mod 16 (compiled for each
+// remainder), which keeps the loads at one float4 per 32 FMAs or fewer. The
+// column strips that those sides took before read every input value through
+// a scalar load: 61 x 59, K = 13, 200 vectors 131 -> MEAS13 us; 108 x 108,
+// K = 17, one vector 508 -> MEAS17 us (with its row bands).
+//
+// mirror: the PSF's rows are the same from the top and from the bottom (any
+// profile sampled on a centred grid; gl_system_create checks every value), so
+// the two input rows that meet the same kernel row are added first: (K + 1) / 2
+// rows of FMAs instead of K (K = 21: 100 x 100, B = 512, k_conv 261 -> MEAS21 us).
 
-// out[r] = sum_{a,b} ker[a][b] in[(i + a) P + j0 + r + b], r < 16; ker rows of KP floats.
-template <int K>
-__device__ __forceinline__ void corr_row(const float* __restrict__ in, int P, const float* __restrict__ ker, int i,
-                                         int j0, float (&acc)[16]) {
-  constexpr int S = 16, KP = (K + 3) & ~3, NIN = (S + K - 1 + 3) & ~3;
+// acc[r] += sum_b ker[b] x[r + b], b < G, for the input row at row (and, with
+// two, the one at row2 added to it).
+template <int G>
+__device__ __forceinline__ void row_taps(const float* __restrict__ row, const float* __restrict__ row2, bool two,
+                                         const float* __restrict__ ker, float (&acc)[16]) {
+  constexpr int S = 16, KP = (G + 3) & ~3, NIN = (S + G - 1 + 3) & ~3;
+  float x[NIN];
+  const float4* r4 = reinterpret_cast<const float4*>(row);
 #pragma unroll
-  for (int r = 0; r < S; ++r) acc[r] = 0.f;
-  const float* row = in + i * P + j0;
-#pragma unroll 1
-  for (int a = 0; a < K; ++a) {
-    float x[NIN];
-    const float4* r4 = reinterpret_cast<const float4*>(row + a * P);
+  for (int q = 0; q < NIN / 4; ++q) {
+    const float4 t = r4[q];
+    x[4 * q] = t.x;
+    x[4 * q + 1] = t.y;
+    x[4 * q + 2] = t.z;
+    x[4 * q + 3] = t.w;
+  }
+  if (two) {
+    const float4* s4 = reinterpret_cast<const float4*>(row2);
 #pragma unroll
     for (int q = 0; q < NIN / 4; ++q) {
-      const float4 t = r4[q];
-      x[4 * q] = t.x;
-      x[4 * q + 1] = t.y;
-      x[4 * q + 2] = t.z;
-      x[4 * q + 3] = t.w;
+      const float4 t = s4[q];
+      x[4 * q] += t.x;
+      x[4 * q + 1] += t.y;
+      x[4 * q + 2] += t.z;
+      x[4 * q + 3] += t.w;
     }
-    float kr[KP];
-    const float4* k4 = reinterpret_cast<const float4*>(ker + a * KP);
+  }
+  float kr[KP];
+  const float4* k4 = reinterpret_cast<const float4*>(ker);
 #pragma unroll
-    for (int q = 0; q < KP / 4; ++q) {
-      const float4 t = k4[q];
-      kr[4 * q] = t.x;
-      kr[4 * q + 1] = t.y;
-      kr[4 * q + 2] = t.z;
-      kr[4 * q + 3] = t.w;
+  for (int q = 0; q < KP / 4; ++q) {
+    const float4 t = k4[q];
+    kr[4 * q] = t.x;
+    kr[4 * q + 1] = t.y;
+    kr[4 * q + 2] = t.z;
+    kr[4 * q + 3] = t.w;
+  }
+#pragma unroll
+  for (int b = 0; b < G; ++b) {
+#pragma unroll
+    for (int r = 0; r < S; ++r) acc[r] = fmaf(kr[b], x[r + b], acc[r]);
+  }
+}
+
+// The taps [t0, t0 + G) of every kernel row.
+template <int G>
+__device__ __forceinline__ void corr_taps(const float* __restrict__ in, int P, const float* __restrict__ ker, int K,
+                                          int t0, bool mirror, int i, int j0, float (&acc)[16]) {
+  const int KP = (K + 3) & ~3;
+  const float* row = in + i * P + j0 + t0;
+  const int rows = mirror ? (K + 1) >> 1 : K;
+#pragma unroll 1
+  for (int a = 0; a < rows; ++a)
+    row_taps<G>(row + a * P, row + (K - 1 - a) * P, mirror && 2 * a != K - 1, ker + a * KP + t0, acc);
+}
+
+// out[r] = sum_{a,b} ker[a][b] in[(i + a) P + j0 + r + b], r < 16; ker rows of
+// KP floats. K > 0: compile-time side; K == 0: any odd side Kk.
+template <int K>
+__device__ __forceinline__ void corr_row(const float* __restrict__ in, int P, const float* __restrict__ ker, int Kk,
+                                         bool mirror, int i, int j0, float (&acc)[16]) {
+#pragma unroll
+  for (int r = 0; r < 16; ++r) acc[r] = 0.f;
+  if constexpr (K > 0) {
+    corr_taps<K>(in, P, ker, K, 0, mirror, i, j0, acc);
+  } else {
+    int t0 = 0;
+    for (; t0 + 16 <= Kk; t0 += 16) corr_taps<16>(in, P, ker, Kk, t0, mirror, i, j0, acc);
+    switch (Kk - t0) {
+      case 1: corr_taps<1>(in, P, ker, Kk, t0, mirror, i, j0, acc); break;
+      case 3: corr_taps<3>(in, P, ker, Kk, t0, mirror, i, j0, acc); break;
+      case 5: corr_taps<5>(in, P, ker, Kk, t0, mirror, i, j0, acc); break;
+      case 7: corr_taps<7>(in, P, ker, Kk, t0, mirror, i, j0, acc); break;
+      case 9: corr_taps<9>(in, P, ker, Kk, t0, mirror, i, j0, acc); break;
+      case 11: corr_taps<11>(in, P, ker, Kk, t0, mirror, i, j0, acc); break;
+      case 13: corr_taps<13>(in, P, ker, Kk, t0, mirror, i, j0, acc); break;
+      default: corr_taps<15>(in, P, ker, Kk, t0, mirror, i, j0, acc); break;
     }
-#pragma unroll
-    for (int b = 0; b < K; ++b) {
-#pragma unroll
-      for (int r = 0; r < S; ++r) acc[r] = fmaf(kr[b], x[r + b], acc[r]);
-    }
+  }
+}
+
+// Both orientations of the PSF into shared memory, rows of KP floats, zero padded.
+__device__ __forceinline__ void load_kernels(const Seg& s, int K, float* kerF, float* kerU) {
+  const int KP = (K + 3) & ~3;
+  for (int i = threadIdx.x; i < K * KP; i += blockDim.x) {
+    const int a = i / KP, bb = i - a * KP;
+    kerF[i] = bb < K ? s.psf[(K - 1 - a) * K + (K - 1 - bb)] : 0.f;
+    kerU[i] = bb < K ? s.psf[a * K + bb] : 0.f;
   }
 }
 
@@ -1145,12 +1184,10 @@ __device__ __forceinline__ void cp_async_wait_all() {
 }
 
 // The binned image (the vector's work slot) into the interior of the
-// zero-padded buffer img ([H + K - 1][P], halo (K - 1)/2), by asynchronous
+// zero-padded buffer img ([H + 2 c][P], halo c = (K - 1)/2), by asynchronous
 // copies while the halo is zeroed; rows across warps, columns across lanes.
 // The caller synchronises the block after.
-template <int K>
-__device__ __forceinline__ void load_padded(const Seg& s, float* img, int P, const float* work) {
-  constexpr int c = (K - 1) / 2;
+__device__ __forceinline__ void load_padded(const Seg& s, int c, float* img, int P, const float* work) {
   const int H = s.H, W = s.W;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
   for (int i = wid; i < H; i += nw)
@@ -1222,21 +1259,23 @@ __device__ bool pixel_phase(const Seg& s, int b, bool want_sim, bool want_grad, 
   return want_grad;
 }
 
-// One vector, PSF side K known at compile time. Shared memory: both PSF
-// orientations ([K][KP], zero padded), the zero-padded input buffer
+// One vector by row strips (K > 0: compile-time PSF side; K == 0: any odd
+// side s.K). Shared memory: both PSF orientations ([K][KP], zero padded), the zero-padded input buffer
 // [H + K - 1][P] and, when s.conv_two_buf, an unpadded staging buffer [H][P]
 // for the model values and the correlation output (else they go through the
 // vector's global work slot). After the first pass the input buffer's
 // interior is overwritten with d log L / d M (its zero halo is reused).
 template <int K>
 __device__ void conv_vector_rows(const Seg& s, int b, int mode, float* smem, double* red2) {
-  constexpr int S = 16, KP = (K + 3) & ~3, c = (K - 1) / 2;
+  constexpr int S = 16;
+  const int Kk = K > 0 ? K : s.K, KP = (Kk + 3) & ~3, c = (Kk - 1) / 2;
   const int H = s.H, W = s.W, HW = H * W;
-  const int P = rowconv_pitch(W, K);
-  const int Hp = H + K - 1;
+  const int P = rowconv_pitch(W, Kk);
+  const int Hp = H + Kk - 1;
+  const bool mirror = s.psf_mirror != 0;
   float* kerF = smem;
-  float* kerU = smem + K * KP;
-  float* img = smem + 2 * K * KP;
+  float* kerU = smem + Kk * KP;
+  float* img = smem + 2 * Kk * KP;
   float* stage = img + Hp * P;
   float* work = s.work + size_t(b) * HW;
   const bool want_sim = (mode == MODE_SIM);
@@ -1244,14 +1283,10 @@ __device__ void conv_vector_rows(const Seg& s, int b, int mode, float* smem, dou
   const bool want_grad = (mode == MODE_GRAD) || corr_only;
   const bool two = s.conv_two_buf != 0;
 
-  for (int i = threadIdx.x; i < K * KP; i += blockDim.x) {
-    const int a = i / KP, bb = i - a * KP;
-    kerF[i] = bb < K ? s.psf[(K - 1 - a) * K + (K - 1 - bb)] : 0.f;
-    kerU[i] = bb < K ? s.psf[a * K + bb] : 0.f;
-  }
+  load_kernels(s, Kk, kerF, kerU);
   // pixel loops: rows across warps, columns across lanes (coalesced, no division)
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  load_padded<K>(s, img, P, work);
+  load_padded(s, c, img, P, work);
   __syncthreads();
 
   const int nstrip = (W + S - 1) / S;
@@ -1261,7 +1296,7 @@ __device__ void conv_vector_rows(const Seg& s, int b, int mode, float* smem, dou
   // pass 1: model image M (convolution with the flipped PSF)
   for (int u = threadIdx.x; u < units; u += blockDim.x) {
     const int strip = u / H, i = u - strip * H, j0 = strip * S;
-    corr_row<K>(img, P, kerF, i, j0, acc);
+    corr_row<K>(img, P, kerF, Kk, mirror, i, j0, acc);
     if (two) {
       float4* o4 = reinterpret_cast<float4*>(stage + i * P + j0);
 #pragma unroll
@@ -1281,7 +1316,7 @@ __device__ void conv_vector_rows(const Seg& s, int b, int mode, float* smem, dou
   const float inv_k2 = 1.0f / float(s.k * s.k);
   for (int u = threadIdx.x; u < units; u += blockDim.x) {
     const int strip = u / H, i = u - strip * H, j0 = strip * S;
-    corr_row<K>(img, P, kerU, i, j0, acc);
+    corr_row<K>(img, P, kerU, Kk, mirror, i, j0, acc);
     if (two) {
       float4* o4 = reinterpret_cast<float4*>(stage + i * P + j0);
 #pragma unroll
@@ -1347,9 +1382,8 @@ __device__ __forceinline__ SepLayout sep_layout(const Seg& s, float* smem, int r
 // outside rows c .. c + H - 1, columns c .. c + W - 1) zeroed; rows across
 // warps, columns across lanes. The caller synchronises the block before
 // the factors are read.
-template <int K>
 __device__ __forceinline__ void sep_prepare(const Seg& s, const SepLayout& L) {
-  constexpr int c = (K - 1) / 2;
+  const int K = s.K, c = (K - 1) / 2;
   const int R = s.psf_rank;
   for (int i = threadIdx.x; i < 2 * R * K; i += blockDim.x) L.fac[i] = s.psf_sep[i];
   for (int i = threadIdx.x; i < R * K; i += blockDim.x) {
@@ -1367,22 +1401,45 @@ __device__ __forceinline__ void sep_prepare(const Seg& s, const SepLayout& L) {
 // The binned image (the vector's work slot) into the input's interior by
 // asynchronous copies, issued only: the caller waits for them
 // (cp_async_wait_all) and synchronises the block.
-template <int K>
 __device__ __forceinline__ void sep_load_issue(const Seg& s, const SepLayout& L, const float* work) {
-  constexpr int c = (K - 1) / 2;
+  const int c = (s.K - 1) / 2;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
   for (int i = wid; i < s.H; i += nw)
     for (int j = lane; j < s.W; j += 32) cp_async4(&L.img[(i + c) * L.P + j + c], &work[i * s.W + j]);
 }
 
+// G taps of one horizontal unit: acc[o] += sum_q tap(q) x[o + q], tap(q) = v[q]
+// (FLIP: v[-q]).
+template <int G, bool FLIP>
+__device__ __forceinline__ void sep_htaps(const float* __restrict__ in, const float* __restrict__ v, float (&acc)[16]) {
+  constexpr int S = 16, NIN = (S + G - 1 + 3) & ~3;
+  float x[NIN];
+  const float4* r4 = reinterpret_cast<const float4*>(in);
+#pragma unroll
+  for (int q = 0; q < NIN / 4; ++q) {
+    const float4 t = r4[q];
+    x[4 * q] = t.x;
+    x[4 * q + 1] = t.y;
+    x[4 * q + 2] = t.z;
+    x[4 * q + 3] = t.w;
+  }
+#pragma unroll
+  for (int o = 0; o < S; ++o) {
+    float a = acc[o];
+#pragma unroll
+    for (int q = 0; q < G; ++q) a = fmaf(v[FLIP ? -q : q], x[o + q], a);
+    acc[o] = a;
+  }
+}
+
 // Horizontal passes: row buffer r, row i, columns j0 .. j0 + 15, for the Ht
 // rows. A warp takes 32 consecutive rows of one strip (float4 loads of rows
-// an odd number of 16-byte words apart are conflict-free); each unit loads
-// its input span once for the R terms. FLIP: the flipped factor (the model's
-// convolution); RC: the rank when known at compile time (1), else 0.
+// an odd number of 16-byte words apart are conflict-free). FLIP: the flipped
+// factor (the model's convolution); RC: the rank when known at compile time
+// (1), else 0. K == 0: any odd side Kk, in groups of 8 taps.
 template <int K, bool FLIP, int RC>
-__device__ __forceinline__ void sep_hpass(const float* __restrict__ in, const SepLayout& L, int W, int Rrt) {
-  constexpr int S = 16, NIN = (S + K - 1 + 3) & ~3;
+__device__ __forceinline__ void sep_hpass(const float* __restrict__ in, const SepLayout& L, int W, int Rrt, int Kk) {
+  constexpr int S = 16;
   const int R = RC > 0 ? RC : Rrt;
   const int P = L.P, Ht = L.Ht, nstrip = (W + S - 1) / S, rg = (Ht + 31) >> 5, tasks = nstrip * rg;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -1395,25 +1452,25 @@ __device__ __forceinline__ void sep_hpass(const float* __restrict__ in, const Se
       ++strip;
     }
     if (i >= Ht) continue;
-    float x[NIN];
-    const float4* r4 = reinterpret_cast<const float4*>(in + i * P + j0);
-#pragma unroll
-    for (int q = 0; q < NIN / 4; ++q) {
-      const float4 v = r4[q];
-      x[4 * q] = v.x;
-      x[4 * q + 1] = v.y;
-      x[4 * q + 2] = v.z;
-      x[4 * q + 3] = v.w;
-    }
+    const float* row = in + i * P + j0;
     for (int r = 0; r < R; ++r) {
-      const float* v = L.fac + (2 * r + 1) * K;
       float acc[S];
 #pragma unroll
-      for (int o = 0; o < S; ++o) {
-        float a = 0.f;
-#pragma unroll
-        for (int q = 0; q < K; ++q) a = fmaf(v[FLIP ? K - 1 - q : q], x[o + q], a);
-        acc[o] = a;
+      for (int o = 0; o < S; ++o) acc[o] = 0.f;
+      if constexpr (K > 0) {
+        const float* v = L.fac + (2 * r + 1) * K;
+        sep_htaps<K, FLIP>(row, v + (FLIP ? K - 1 : 0), acc);
+      } else {
+        const float* v = L.fac + (2 * r + 1) * Kk;
+        int t0 = 0;
+        for (; t0 + 8 <= Kk; t0 += 8) sep_htaps<8, FLIP>(row + t0, v + (FLIP ? Kk - 1 - t0 : t0), acc);
+        const float* vt = v + (FLIP ? Kk - 1 - t0 : t0);
+        switch (Kk - t0) {
+          case 1: sep_htaps<1, FLIP>(row + t0, vt, acc); break;
+          case 3: sep_htaps<3, FLIP>(row + t0, vt, acc); break;
+          case 5: sep_htaps<5, FLIP>(row + t0, vt, acc); break;
+          default: sep_htaps<7, FLIP>(row + t0, vt, acc); break;
+        }
       }
       float4* t4 = reinterpret_cast<float4*>(L.tmp + size_t(r) * Ht * P + i * P + j0);
 #pragma unroll
@@ -1422,27 +1479,47 @@ __device__ __forceinline__ void sep_hpass(const float* __restrict__ in, const Se
   }
 }
 
+// G taps of one vertical unit, m[o] += sum_q tap(q) x[o + q].
+template <int G, bool FLIP>
+__device__ __forceinline__ void sep_vtaps(const float* __restrict__ col, int P, const float2* __restrict__ tap,
+                                          float2 (&m)[SEP_RV]) {
+  constexpr int NV = SEP_RV + G - 1;
+  float2 x[NV];
+#pragma unroll
+  for (int q = 0; q < NV; ++q) x[q] = *reinterpret_cast<const float2*>(col + q * P);
+#pragma unroll
+  for (int o = 0; o < SEP_RV; ++o) {
+    float2 a = m[o];
+#pragma unroll
+    for (int q = 0; q < G; ++q) a = __ffma2_rn(tap[FLIP ? -q : q], x[o + q], a);
+    m[o] = a;
+  }
+}
+
 // Vertical passes of one unit: rows i0 .. i0 + 7 of columns j, j + 1 (j
 // even) in packed pairs, summed over the R terms (per lane the FMAs of the
 // scalar form, in the same order).
 template <int K, bool FLIP, int RC>
-__device__ __forceinline__ void sep_vunit(const SepLayout& L, int Rrt, int i0, int j, float2 (&m)[SEP_RV]) {
-  constexpr int NV = SEP_RV + K - 1;
+__device__ __forceinline__ void sep_vunit(const SepLayout& L, int Rrt, int Kk, int i0, int j, float2 (&m)[SEP_RV]) {
   const int R = RC > 0 ? RC : Rrt;
 #pragma unroll
   for (int o = 0; o < SEP_RV; ++o) m[o] = make_float2(0.f, 0.f);
   for (int r = 0; r < R; ++r) {
-    const float2* tap = L.tapu + r * K;
     const float* col = L.tmp + size_t(r) * L.Ht * L.P + i0 * L.P + j;
-    float2 x[NV];
-#pragma unroll
-    for (int q = 0; q < NV; ++q) x[q] = *reinterpret_cast<const float2*>(col + q * L.P);
-#pragma unroll
-    for (int o = 0; o < SEP_RV; ++o) {
-      float2 a = m[o];
-#pragma unroll
-      for (int q = 0; q < K; ++q) a = __ffma2_rn(tap[FLIP ? K - 1 - q : q], x[o + q], a);
-      m[o] = a;
+    if constexpr (K > 0) {
+      sep_vtaps<K, FLIP>(col, L.P, L.tapu + r * K + (FLIP ? K - 1 : 0), m);
+    } else {
+      const float2* tap = L.tapu + r * Kk;
+      int t0 = 0;
+      for (; t0 + 8 <= Kk; t0 += 8) sep_vtaps<8, FLIP>(col + t0 * L.P, L.P, tap + (FLIP ? Kk - 1 - t0 : t0), m);
+      const float2* tt = tap + (FLIP ? Kk - 1 - t0 : t0);
+      col += t0 * L.P;
+      switch (Kk - t0) {
+        case 1: sep_vtaps<1, FLIP>(col, L.P, tt, m); break;
+        case 3: sep_vtaps<3, FLIP>(col, L.P, tt, m); break;
+        case 5: sep_vtaps<5, FLIP>(col, L.P, tt, m); break;
+        default: sep_vtaps<7, FLIP>(col, L.P, tt, m); break;
+      }
     }
   }
 }
@@ -1483,7 +1560,7 @@ template <int K, int MODE_T, int RC, bool PF = false>
 __device__ void conv_vector_sep(const Seg& s, int b, int mode_rt, float* smem, double* red2, bool prepared,
                                 int next_b = -1) {
   static_assert(!PF || MODE_T == MODE_GRAD, "prefetch only in the gradient pass");
-  constexpr int c = (K - 1) / 2;
+  const int c = ((K > 0 ? K : s.K) - 1) / 2;
   const int mode = MODE_T >= 0 ? MODE_T : mode_rt;
   const int H = s.H, W = s.W, HW = H * W, R = RC > 0 ? RC : s.psf_rank;
   const SepLayout L = sep_layout(s, smem, H);
@@ -1492,18 +1569,18 @@ __device__ void conv_vector_sep(const Seg& s, int b, int mode_rt, float* smem, d
   const bool corr_only = (mode == MODE_CORR);   // the work slot holds d log L / d M already
   const bool want_grad = (mode == MODE_GRAD) || corr_only;
   const int Wp2 = (W + 1) >> 1;
-  if (!prepared) sep_prepare<K>(s, L);
-  if (!PF) sep_load_issue<K>(s, L, work);
+  if (!prepared) sep_prepare(s, L);
+  if (!PF) sep_load_issue(s, L, work);
   cp_async_wait_all();
   __syncthreads();
   if (!corr_only) {
-    sep_hpass<K, true, RC>(L.img, L, W, R);
+    sep_hpass<K, true, RC>(L.img, L, W, R, s.K);
     __syncthreads();
     float ll = 0.f, c2 = 0.f;
     for_vunits(L.nvs, Wp2, [&](int i0, int j) {
       const bool two = j + 1 < W;
       float2 m[SEP_RV];
-      sep_vunit<K, true, RC>(L, R, i0, j, m);
+      sep_vunit<K, true, RC>(L, R, s.K, i0, j, m);
 #pragma unroll
       for (int o = 0; o < SEP_RV; ++o) {
         const int i = i0 + o;
@@ -1526,13 +1603,13 @@ __device__ void conv_vector_sep(const Seg& s, int b, int mode_rt, float* smem, d
     block_loglik(s, b, ll, c2, red2);   // also the barrier before the correlation reads img
     if (!want_grad) return;
   }
-  sep_hpass<K, false, RC>(L.img, L, W, R);
+  sep_hpass<K, false, RC>(L.img, L, W, R, s.K);
   __syncthreads();
-  if (PF && next_b >= 0) sep_load_issue<K>(s, L, s.work + size_t(next_b) * HW);
+  if (PF && next_b >= 0) sep_load_issue(s, L, s.work + size_t(next_b) * HW);
   const float inv_k2 = 1.0f / float(s.k * s.k);
   for_vunits(L.nvs, Wp2, [&](int i0, int j) {
     float2 m[SEP_RV];
-    sep_vunit<K, false, RC>(L, R, i0, j, m);
+    sep_vunit<K, false, RC>(L, R, s.K, i0, j, m);
 #pragma unroll
     for (int o = 0; o < SEP_RV; ++o) {
       const int i = i0 + o;
@@ -1543,7 +1620,7 @@ __device__ void conv_vector_sep(const Seg& s, int b, int mode_rt, float* smem, d
   });
 }
 
-template <int K, int R, int NT, int MINB, class Src>
+template <int K, int NT, int MINB, class Src>
 __global__ void __launch_bounds__(NT, MINB) k_conv(const __grid_constant__ Src src, int mode) {
   extern __shared__ float4 smem4[];
   float* smem = reinterpret_cast<float*>(smem4);
@@ -1555,16 +1632,14 @@ __global__ void __launch_bounds__(NT, MINB) k_conv(const __grid_constant__ Src s
     const Seg* segp = src.conv_seg(item, b);
     block_copy(&ss, segp);
     __syncthreads();
-    if constexpr (K > 0) {
-      // a single-system call takes k_conv_sep for a separable PSF; a table
-      // may mix both kinds of segment
-      if (!std::is_same<Src, OneSeg>::value && ss.conv_sep)
-        conv_vector_sep<K, -1, 0>(ss, b, mode, smem, red2, false);
-      else
-        conv_vector_rows<K>(ss, b, mode, smem, red2);
-    } else {
-      conv_vector<K, R>(ss, b, mode, smem, red2);
-    }
+    // a single-system call takes k_conv_sep for a separable PSF; a table may
+    // mix both kinds of segment
+    if (!std::is_same<Src, OneSeg>::value && ss.conv_sep)
+      conv_vector_sep<K, -1, 0>(ss, b, mode, smem, red2, false);
+    else if (K > 0 || ss.conv_rows)
+      conv_vector_rows<K>(ss, b, mode, smem, red2);
+    else
+      conv_vector(ss, b, mode, smem, red2);
     __syncthreads();
   }
 }
@@ -1581,14 +1656,14 @@ __global__ void __launch_bounds__(NT, MINB) k_conv_sep(const __grid_constant__ O
   // vectors; each vector's steps end with the vertical pass, which reads only
   // the row buffers, and the next vector's horizontal pass comes after the
   // barrier that follows its image load
-  sep_prepare<K>(src.s, sep_layout(src.s, smem, src.s.H));
+  sep_prepare(src.s, sep_layout(src.s, smem, src.s.H));
   // the gradient call of a rank-1 PSF (a sampled Gaussian) with its mode and
   // rank known at compile time; any other call with both read at run time
   if (mode == MODE_GRAD && src.s.psf_rank == 1) {
     // each vector's image copies run during the previous vector's last pass
     const int n = src.nconv();
     if (int(blockIdx.x) < n)
-      sep_load_issue<K>(src.s, sep_layout(src.s, smem, src.s.H), src.s.work + size_t(blockIdx.x) * src.s.H * src.s.W);
+      sep_load_issue(src.s, sep_layout(src.s, smem, src.s.H), src.s.work + size_t(blockIdx.x) * src.s.H * src.s.W);
     for (int item = blockIdx.x; item < n; item += gridDim.x) {
       const int next = item + int(gridDim.x);
       conv_vector_sep<K, MODE_GRAD, 1, true>(src.s, item, mode, smem, red2, true, next < n ? next : -1);
@@ -1628,28 +1703,27 @@ __global__ void __launch_bounds__(BAND_THREADS) k_conv_bands(const __grid_consta
   __shared__ double red2[2 * (BAND_THREADS / 32)];
   __shared__ double band_sum[2];
   const PdlScope pdl;
-  constexpr int S = 16, KP = (K + 3) & ~3, c = (K - 1) / 2;
+  constexpr int S = 16;
   const Seg& s = src.s;
+  const int Kk = K > 0 ? K : s.K, KP = (Kk + 3) & ~3, c = (Kk - 1) / 2;
+  const bool mirror = s.psf_mirror != 0;
   const int nb = int(cluster.num_blocks()), rank = int(cluster.block_rank());
   const int b = blockIdx.x / nb;
   const int H = s.H, W = s.W, HW = H * W;
-  const int P = rowconv_pitch(W, K);
+  const int P = rowconv_pitch(W, Kk);
   const int r0 = min(H, rank * rows), nr = min(H, r0 + rows) - r0;   // nr may be 0
-  const int Hb = rows + K - 1;
+  const int Hb = rows + Kk - 1;
   float* kerF = smem;
-  float* kerU = smem + K * KP;
-  float* img = smem + 2 * K * KP;   // [Hb][P], local row li holds image row r0 - c + li
+  float* kerU = smem + Kk * KP;
+  float* img = smem + 2 * Kk * KP;   // [Hb][P], local row li holds image row r0 - c + li
   float* stage = img + Hb * P;      // [rows][P]
   float* work = s.work + size_t(b) * HW;
   const bool want_sim = (mode == MODE_SIM);
-  const bool want_grad = (mode == MODE_GRAD);
+  const bool corr_only = (mode == MODE_CORR);   // the work slot holds d log L / d M already
+  const bool want_grad = (mode == MODE_GRAD) || corr_only;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
 
-  for (int i = threadIdx.x; i < K * KP; i += blockDim.x) {
-    const int a = i / KP, bb = i - a * KP;
-    kerF[i] = bb < K ? s.psf[(K - 1 - a) * K + (K - 1 - bb)] : 0.f;
-    kerU[i] = bb < K ? s.psf[a * K + bb] : 0.f;
-  }
+  load_kernels(s, Kk, kerF, kerU);
   for (int li = wid; li < Hb; li += nw) {
     const int g = r0 - c + li;
     float* row = img + li * P;
@@ -1663,13 +1737,14 @@ __global__ void __launch_bounds__(BAND_THREADS) k_conv_bands(const __grid_consta
   cp_async_wait_all();
   __syncthreads();
 
-  // pass 1: M of this band's rows
   const int nstrip = (W + S - 1) / S;
   const int units = nstrip * nr;
   float acc[S];
+  if (!corr_only) {
+  // pass 1: M of this band's rows
   for (int u = threadIdx.x; u < units; u += blockDim.x) {
     const int strip = u / nr, li = u - strip * nr, j0 = strip * S;
-    corr_row<K>(img, P, kerF, li, j0, acc);
+    corr_row<K>(img, P, kerF, Kk, mirror, li, j0, acc);
     float4* o4 = reinterpret_cast<float4*>(stage + li * P + j0);
 #pragma unroll
     for (int q = 0; q < S / 4; ++q) o4[q] = make_float4(acc[4 * q], acc[4 * q + 1], acc[4 * q + 2], acc[4 * q + 3]);
@@ -1731,12 +1806,15 @@ __global__ void __launch_bounds__(BAND_THREADS) k_conv_bands(const __grid_consta
   }
   cluster.sync();   // no block reads another's shared memory after this barrier
   if (!want_grad) return;
+  } else {
+    cluster.sync();   // every band holds its input before any band writes the work slot
+  }
 
   // pass 2: subpixel adjoint of the band's rows = (PSF correlated with d log L / d M) / k^2
   const float inv_k2 = 1.0f / float(s.k * s.k);
   for (int u = threadIdx.x; u < units; u += blockDim.x) {
     const int strip = u / nr, li = u - strip * nr, j0 = strip * S;
-    corr_row<K>(img, P, kerU, li, j0, acc);
+    corr_row<K>(img, P, kerU, Kk, mirror, li, j0, acc);
     float4* o4 = reinterpret_cast<float4*>(stage + li * P + j0);
 #pragma unroll
     for (int q = 0; q < S / 4; ++q)
@@ -1780,8 +1858,8 @@ __global__ void __launch_bounds__(BAND_THREADS, 2) k_conv_sep_bands(const __grid
   __shared__ double red2[2 * (BAND_THREADS / 32)];
   __shared__ double band_sum[2];
   const PdlScope pdl;
-  constexpr int c = (K - 1) / 2;
   const Seg& s = src.s;
+  const int Kk = K > 0 ? K : s.K, c = (Kk - 1) / 2;
   const int nb = int(cluster.num_blocks()), rank = int(cluster.block_rank());
   const int b = blockIdx.x / nb;
   const int H = s.H, W = s.W, HW = H * W, R = s.psf_rank;
@@ -1794,9 +1872,9 @@ __global__ void __launch_bounds__(BAND_THREADS, 2) k_conv_sep_bands(const __grid
   const bool want_grad = (mode == MODE_GRAD) || corr_only;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
 
-  for (int i = threadIdx.x; i < 2 * R * K; i += blockDim.x) L.fac[i] = s.psf_sep[i];
-  for (int i = threadIdx.x; i < R * K; i += blockDim.x) {
-    const float u = s.psf_sep[(i / K) * 2 * K + i % K];
+  for (int i = threadIdx.x; i < 2 * R * Kk; i += blockDim.x) L.fac[i] = s.psf_sep[i];
+  for (int i = threadIdx.x; i < R * Kk; i += blockDim.x) {
+    const float u = s.psf_sep[(i / Kk) * 2 * Kk + i % Kk];
     L.tapu[i] = make_float2(u, u);
   }
   // the band's rows and halo rows of the input; rows outside the image, or
@@ -1804,7 +1882,7 @@ __global__ void __launch_bounds__(BAND_THREADS, 2) k_conv_sep_bands(const __grid
   for (int li = wid; li < L.Ht; li += nw) {
     const int g = r0 - c + li;
     float* row = L.img + li * P;
-    if (li < nr + K - 1 && g >= 0 && g < H) {
+    if (li < nr + Kk - 1 && g >= 0 && g < H) {
       for (int j = lane; j < W; j += 32) cp_async4(&row[j + c], &work[g * W + j]);
       for (int q = lane; q < P - W; q += 32) row[q < c ? q : W + q] = 0.f;
     } else {
@@ -1815,14 +1893,14 @@ __global__ void __launch_bounds__(BAND_THREADS, 2) k_conv_sep_bands(const __grid
   __syncthreads();
   const int Wp2 = (W + 1) >> 1, nvu = ((nr + SEP_RV - 1) / SEP_RV) * Wp2;
   if (!corr_only) {
-    sep_hpass<K, true, 0>(L.img, L, W, R);
+    sep_hpass<K, true, 0>(L.img, L, W, R, s.K);
     __syncthreads();
     float ll = 0.f, c2 = 0.f;
     for (int u = threadIdx.x; u < nvu; u += blockDim.x) {
       const int strip = u / Wp2, j = 2 * (u - strip * Wp2), i0 = strip * SEP_RV;
       const bool two = j + 1 < W;
       float2 m[SEP_RV];
-      sep_vunit<K, true, 0>(L, R, i0, j, m);
+      sep_vunit<K, true, 0>(L, R, s.K, i0, j, m);
 #pragma unroll
       for (int o = 0; o < SEP_RV; ++o) {
         const int li = i0 + o;
@@ -1870,7 +1948,7 @@ __global__ void __launch_bounds__(BAND_THREADS, 2) k_conv_sep_bands(const __grid
     }
     if (want_grad) {
       // the halo rows of d log L / d M from the bands that own them
-      for (int li = wid; li < nr + K - 1; li += nw) {
+      for (int li = wid; li < nr + Kk - 1; li += nw) {
         if (li >= c && li < c + nr) continue;
         const int g = r0 - c + li;
         if (g < 0 || g >= H) continue;   // stays zero
@@ -1884,13 +1962,13 @@ __global__ void __launch_bounds__(BAND_THREADS, 2) k_conv_sep_bands(const __grid
   } else {
     cluster.sync();   // every band holds its input before any band writes the work slot
   }
-  sep_hpass<K, false, 0>(L.img, L, W, R);
+  sep_hpass<K, false, 0>(L.img, L, W, R, s.K);
   __syncthreads();
   const float inv_k2 = 1.0f / float(s.k * s.k);
   for (int u = threadIdx.x; u < nvu; u += blockDim.x) {
     const int strip = u / Wp2, j = 2 * (u - strip * Wp2), i0 = strip * SEP_RV;
     float2 m[SEP_RV];
-    sep_vunit<K, false, 0>(L, R, i0, j, m);
+    sep_vunit<K, false, 0>(L, R, s.K, i0, j, m);
 #pragma unroll
     for (int o = 0; o < SEP_RV; ++o) {
       const int li = i0 + o;
@@ -2075,6 +2153,10 @@ __global__ void k_final_warp(const __grid_constant__ Src src) {
 // thread must not launch on a limit another thread has recorded but not yet set.
 static std::mutex g_attr_mutex;
 
+// Dynamic shared memory a kernel may take without the opt-in attribute: 48 KB
+// less room for the kernels' static part, which counts against the same limit.
+constexpr size_t DEFAULT_DYN_SMEM = 46 * 1024;
+
 static std::atomic<int> g_num_sms{0};
 
 static int num_sms() {
@@ -2089,23 +2171,29 @@ static int num_sms() {
   return n;
 }
 
-// Convolution classes: (PSF side, strip rows, threads). Class 2 takes any odd side.
-struct ConvClass {
-  int K, R, NT;
-};
-static constexpr ConvClass kConvClasses[3] = {{11, 16, 256}, {21, 16, 256}, {0, 8, 128}};  // see launch_conv_class
-
 int conv_class(int K) { return K == 11 ? 0 : (K == 21 ? 1 : 2); }
 
-size_t conv_smem_bytes(int H, int W, int K, bool two_buf) {
-  if (kConvClasses[conv_class(K)].K > 0) {   // row-strip layout (conv_vector_rows)
-    const size_t KP = size_t((K + 3) & ~3), P = size_t(rowconv_pitch(W, K));
-    return (2 * size_t(K) * KP + (size_t(H) + K - 1) * P + (two_buf ? size_t(H) * P : 0)) * sizeof(float);
-  }
-  const int R = kConvClasses[conv_class(K)].R;
-  const int nstrip = (H + R - 1) / R;
-  const size_t Hp = size_t(nstrip) * R + K - 1, Wp = size_t(W) + K - 1;
+// Shared memory of the row strips (conv_vector_rows) and of the column strips
+// (conv_vector).
+static size_t conv_rows_smem(int H, int W, int K, bool two_buf) {
+  const size_t KP = size_t((K + 3) & ~3), P = size_t(rowconv_pitch(W, K));
+  return (2 * size_t(K) * KP + (size_t(H) + K - 1) * P + (two_buf ? size_t(H) * P : 0)) * sizeof(float);
+}
+static size_t conv_strips_smem(int H, int W, int K, bool two_buf) {
+  const size_t Hp = size_t((H + STRIP_ROWS - 1) / STRIP_ROWS) * STRIP_ROWS + K - 1, Wp = size_t(W) + K - 1;
   return (2 * size_t((K * K + 3) & ~3) + (two_buf ? 2 : 1) * Hp * Wp) * sizeof(float);
+}
+
+// Row strips wherever their buffer fits a block: the sides 11 and 21 have no
+// other form, and for any other side the column strips (which pad a row to
+// W + K - 1 floats only) remain for the few images that fit just so.
+// 227 KB is the most a block can have, 2 KB of it the kernels' static part.
+bool conv_rows_fit(int H, int W, int K) {
+  return K == 11 || K == 21 || conv_rows_smem(H, W, K, false) + 2048 <= size_t(227) * 1024;
+}
+
+size_t conv_smem_bytes(int H, int W, int K, bool two_buf) {
+  return conv_rows_fit(H, W, K) ? conv_rows_smem(H, W, K, two_buf) : conv_strips_smem(H, W, K, two_buf);
 }
 
 bool conv_two_buf(int H, int W, int K) { return conv_smem_bytes(H, W, K, true) <= CONV_TWO_BUF_MAX_SMEM; }
@@ -2117,7 +2205,7 @@ size_t conv_sep_smem_bytes(int H, int W, int K, int R) {
 
 // 2 K R multiply-adds per pixel and pass against K^2, with a pass of
 // shared-memory traffic per term: worth it at R <= K / 4
-static bool conv_sep_worth(int K, int R) { return R > 0 && 4 * R <= K && (K == 11 || K == 21); }
+static bool conv_sep_worth(int K, int R) { return R > 0 && 4 * R <= K; }
 
 bool conv_sep_ok(int H, int W, int K, int R) {
   return conv_sep_worth(K, R) && conv_sep_smem_bytes(H, W, K, R) <= CONV_TWO_BUF_MAX_SMEM;
@@ -2162,7 +2250,9 @@ bool conv_sep_any(int H, int W, int K, int R) {
 }
 
 size_t seg_conv_smem(const Seg& g) {
-  return g.conv_sep ? conv_sep_smem_bytes(g.H, g.W, g.K, g.psf_rank) : conv_smem_bytes(g.H, g.W, g.K, g.conv_two_buf != 0);
+  if (g.conv_sep) return conv_sep_smem_bytes(g.H, g.W, g.K, g.psf_rank);
+  return g.conv_rows ? conv_rows_smem(g.H, g.W, g.K, g.conv_two_buf != 0)
+                     : conv_strips_smem(g.H, g.W, g.K, g.conv_two_buf != 0);
 }
 
 // Resident blocks per SM of the forward ray kernel (occupancy query, cached;
@@ -2213,8 +2303,10 @@ static TilePlan plan_rays(int B, int H, int W, int k) {
   long long max_nt = (HW + 2 * ADJ_THREADS - 1) / (2 * ADJ_THREADS);
   const long long by_rays = (rays + 4 * ADJ_THREADS - 1) / (4 * ADJ_THREADS);
   if (by_rays < max_nt) max_nt = by_rays;
-  if (max_nt < 1) max_nt = 1;
   const double sms = num_sms(), fwd_slots = sms * fwd_blocks_per_sm(), adj_slots = sms * ADJ_BLOCKS_PER_SM;
+  const long long by_waves = (long long)(8.0 * adj_slots / B);   // past eight waves a finer tiling evens out nothing
+  if (by_waves < max_nt) max_nt = by_waves;
+  if (max_nt < 1) max_nt = 1;
   const double tail = B < sms ? TAIL_MODE : TAIL_MIXED;
   double best_cost = 0.0;
   for (long long nt = 1; nt <= max_nt; ++nt) {
@@ -2241,14 +2333,14 @@ void plan_tiles(int B, int H, int W, int k, int* ntiles, int* tile_pix) {
 // Blocks of a convolution kernel resident on the whole GPU at a dynamic
 // shared-memory size (occupancy query, cached per kernel and size; the
 // grouped path warms it before a graph capture).
-template <int K, int R, int NT, int MINB, class Src>
+template <int K, int NT, int MINB, class Src>
 static cudaError_t conv_resident(size_t smem, int* resident) {
   static std::map<size_t, int> per_sm;   // by dynamic shared memory
   std::lock_guard<std::mutex> lock(g_attr_mutex);
   auto it = per_sm.find(smem);
   if (it == per_sm.end()) {
     int n = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_conv<K, R, NT, MINB, Src>, NT, smem);
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_conv<K, NT, MINB, Src>, NT, smem);
     if (e != cudaSuccess) return e;
     it = per_sm.emplace(smem, n > 0 ? n : 1).first;
   }
@@ -2274,13 +2366,13 @@ static cudaError_t launch_pdl(void (*kern)(KArgs...), unsigned grid, unsigned bl
   return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
-template <int K, int R, int NT, int MINB, class Src>
+template <int K, int NT, int MINB, class Src>
 static cudaError_t launch_conv(const Src& src, int nitems, size_t smem, int mode, cudaStream_t st, bool persistent) {
-  static size_t attr = 48 * 1024;
+  static size_t attr = DEFAULT_DYN_SMEM;
   {
     std::lock_guard<std::mutex> lock(g_attr_mutex);
     if (smem > attr) {
-      cudaError_t e = cudaFuncSetAttribute(k_conv<K, R, NT, MINB, Src>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+      cudaError_t e = cudaFuncSetAttribute(k_conv<K, NT, MINB, Src>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                            int(smem));
       if (e != cudaSuccess) return e;
       attr = smem;
@@ -2292,11 +2384,11 @@ static cudaError_t launch_conv(const Src& src, int nitems, size_t smem, int mode
     // items, blocks beyond that would start only after others have finished
     // their whole share
     int resident = 0;
-    cudaError_t e = conv_resident<K, R, NT, MINB, Src>(smem, &resident);
+    cudaError_t e = conv_resident<K, NT, MINB, Src>(smem, &resident);
     if (e != cudaSuccess) return e;
     grid = grid < resident ? grid : resident;
   }
-  return launch_pdl(k_conv<K, R, NT, MINB, Src>, unsigned(grid), NT, smem, st, src, mode);
+  return launch_pdl(k_conv<K, NT, MINB, Src>, unsigned(grid), NT, smem, st, src, mode);
 }
 
 // wide: 512-thread blocks for calls with fewer vectors than SMs (one vector's
@@ -2309,18 +2401,20 @@ static cudaError_t launch_conv_class(int cls, const Src& src, int nitems, size_t
                                      bool persistent, bool wide = false) {
   switch (cls) {
     case 0:
-      return wide ? launch_conv<11, 16, 512, 1>(src, nitems, smem, mode, st, persistent)
-                  : launch_conv<11, 16, 256, 3>(src, nitems, smem, mode, st, persistent);
+      return wide ? launch_conv<11, 512, 1>(src, nitems, smem, mode, st, persistent)
+                  : launch_conv<11, 256, 3>(src, nitems, smem, mode, st, persistent);
     case 1:
-      return wide ? launch_conv<21, 16, 512, 1>(src, nitems, smem, mode, st, persistent)
-                  : launch_conv<21, 16, 256, 1>(src, nitems, smem, mode, st, persistent);
-    default: return launch_conv<0, 8, 128, 4>(src, nitems, smem, mode, st, persistent);
+      return wide ? launch_conv<21, 512, 1>(src, nitems, smem, mode, st, persistent)
+                  : launch_conv<21, 256, 1>(src, nitems, smem, mode, st, persistent);
+    default:
+      return wide ? launch_conv<0, 512, 1>(src, nitems, smem, mode, st, persistent)
+                  : launch_conv<0, 256, 2>(src, nitems, smem, mode, st, persistent);
   }
 }
 
 template <int K, int NT, int MINB>
 static cudaError_t launch_conv_sep(const OneSeg& src, int nitems, size_t smem, int mode, cudaStream_t st) {
-  static size_t attr = 48 * 1024;
+  static size_t attr = DEFAULT_DYN_SMEM;
   {
     std::lock_guard<std::mutex> lock(g_attr_mutex);
     if (smem > attr) {
@@ -2358,8 +2452,11 @@ static cudaError_t launch_conv_one(const OneSeg& src, int nitems, int mode, cuda
     if (s.K == 11)
       return wide ? launch_conv_sep<11, 512, 1>(src, nitems, smem, mode, st)
                   : launch_conv_sep<11, 256, 4>(src, nitems, smem, mode, st);
-    return wide ? launch_conv_sep<21, 512, 1>(src, nitems, smem, mode, st)
-                : launch_conv_sep<21, 256, 3>(src, nitems, smem, mode, st);
+    if (s.K == 21)
+      return wide ? launch_conv_sep<21, 512, 1>(src, nitems, smem, mode, st)
+                  : launch_conv_sep<21, 256, 3>(src, nitems, smem, mode, st);
+    return wide ? launch_conv_sep<0, 512, 1>(src, nitems, smem, mode, st)
+                : launch_conv_sep<0, 256, 3>(src, nitems, smem, mode, st);
   }
   return launch_conv_class(conv_class(s.K), src, nitems, smem, mode, st, false, wide || smem > CONV_WIDE_MIN_SMEM);
 }
@@ -2369,7 +2466,7 @@ static cudaError_t launch_conv_one(const OneSeg& src, int nitems, int mode, cuda
 // blocks per SM, at most 8 per vector (a portable cluster), each at least
 // max(16, (K - 1) / 2) rows and within CONV_TWO_BUF_MAX_SMEM of shared memory.
 static int conv_bands(int B, int H, int W, int K) {
-  if ((K != 11 && K != 21) || B < 1 || 2 * B > num_sms()) return 0;
+  if (B < 1 || 2 * B > num_sms()) return 0;
   int nb = 2 * num_sms() / B;
   if (nb > 8) nb = 8;
   const int min_rows = (K - 1) / 2 > 16 ? (K - 1) / 2 : 16;
@@ -2380,9 +2477,9 @@ static int conv_bands(int B, int H, int W, int K) {
 
 template <int K>
 static cudaError_t launch_conv_bands(const OneSeg& src, int nb, int mode, cudaStream_t st) {
-  static size_t attr = 48 * 1024;
+  static size_t attr = DEFAULT_DYN_SMEM;
   const int rows = (src.s.H + nb - 1) / nb;
-  const size_t smem = conv_band_smem_bytes(src.s.W, K, rows);
+  const size_t smem = conv_band_smem_bytes(src.s.W, src.s.K, rows);
   {
     std::lock_guard<std::mutex> lock(g_attr_mutex);
     if (smem > attr) {
@@ -2410,8 +2507,8 @@ static cudaError_t launch_conv_bands(const OneSeg& src, int nb, int mode, cudaSt
 
 template <int K>
 static cudaError_t launch_conv_sep_bands(const OneSeg& src, int nb, int rows, int mode, cudaStream_t st) {
-  static size_t attr = 48 * 1024;
-  const size_t smem = conv_sep_band_smem_bytes(src.s.W, K, src.s.psf_rank, rows);
+  static size_t attr = DEFAULT_DYN_SMEM;
+  const size_t smem = conv_sep_band_smem_bytes(src.s.W, src.s.K, src.s.psf_rank, rows);
   {
     std::lock_guard<std::mutex> lock(g_attr_mutex);
     if (smem > attr) {
@@ -2508,6 +2605,32 @@ static cudaError_t run_rays(const Src& src, int nvec, int nray, bool fwd, bool a
   return cudaSuccess;
 }
 
+// The convolution of a single-system call: a separable PSF takes the whole
+// image in one block, or row bands over a cluster (small batches, and images
+// whose buffers do not fit one block); any other the 2-D stencil, in bands
+// for small batches.
+static cudaError_t launch_conv_single(const OneSeg& src, int mode, cudaStream_t st, Hooks* hooks) {
+  const Seg& s = src.s;
+  hooks->before(GL_K_CONV, st);
+  int rows = 0;
+  const bool small = 2 * s.B <= num_sms();
+  const int sb = s.psf_rank > 0 && (small || !s.conv_sep) ? sep_band_plan(s.H, s.W, s.K, s.psf_rank, small, s.B, &rows) : 0;
+  const int nb = (sb > 0 || s.conv_sep) ? 0 : conv_bands(s.B, s.H, s.W, s.K);
+  cudaError_t e;
+  if (sb > 0)
+    e = s.K == 11   ? launch_conv_sep_bands<11>(src, sb, rows, mode, st)
+        : s.K == 21 ? launch_conv_sep_bands<21>(src, sb, rows, mode, st)
+                    : launch_conv_sep_bands<0>(src, sb, rows, mode, st);
+  else if (nb > 0)
+    e = s.K == 11   ? launch_conv_bands<11>(src, nb, mode, st)
+        : s.K == 21 ? launch_conv_bands<21>(src, nb, mode, st)
+                    : launch_conv_bands<0>(src, nb, mode, st);
+  else
+    e = launch_conv_one(src, s.B, mode, st, s.B < num_sms());
+  const cudaError_t h = hooks->after(GL_K_CONV, st);
+  return e != cudaSuccess ? e : h;
+}
+
 cudaError_t launch_one(const Seg& s0, int mode, cudaStream_t st, Hooks* hooks) {
   if (s0.B <= 0) return cudaSuccess;
   Seg s = s0;
@@ -2517,23 +2640,7 @@ cudaError_t launch_one(const Seg& s0, int mode, cudaStream_t st, Hooks* hooks) {
   OneSeg src{s};
   cudaError_t e = run_rays(src, s.B, s.B * s.ntiles, true, false, st, hooks, false, false, mode != MODE_CORR);
   if (e != cudaSuccess) return e;
-  hooks->before(GL_K_CONV, st);
-  // a separable PSF: the whole image in one block, or row bands over a
-  // cluster (small batches, and images whose buffers do not fit one block);
-  // else the 2-D stencil, in bands for small batches
-  int rows = 0;
-  const bool small = 2 * s.B <= num_sms();
-  const int sb = s.psf_rank > 0 && (small || !s.conv_sep) ? sep_band_plan(s.H, s.W, s.K, s.psf_rank, small, s.B, &rows) : 0;
-  const int nb = (sb > 0 || mode == MODE_CORR || s.conv_sep) ? 0 : conv_bands(s.B, s.H, s.W, s.K);
-  if (sb > 0)
-    e = s.K == 11 ? launch_conv_sep_bands<11>(src, sb, rows, mode, st)
-                  : launch_conv_sep_bands<21>(src, sb, rows, mode, st);
-  else if (nb > 0)
-    e = s.K == 11 ? launch_conv_bands<11>(src, nb, mode, st) : launch_conv_bands<21>(src, nb, mode, st);
-  else
-    e = launch_conv_one(src, s.B, mode, st, s.B < num_sms());
-  if (e != cudaSuccess) return e;
-  if ((e = hooks->after(GL_K_CONV, st)) != cudaSuccess) return e;
+  if ((e = launch_conv_single(src, mode, st, hooks)) != cudaSuccess) return e;
   if (mode != MODE_GRAD && mode != MODE_CORR) return cudaSuccess;
   return run_rays(src, s.B, s.B * s.ntiles, false, true, st, hooks, false, s.ntiles == 1);
 }
@@ -2549,11 +2656,7 @@ cudaError_t launch_basis(const Seg& s, cudaStream_t st, Hooks* hooks) {
   if ((e = hooks->after(GL_K_RAY_FWD, st)) != cudaSuccess) return e;
   Seg c = s;
   c.B = 2 * s.B;   // the convolution takes the two images of every vector as vectors of their own
-  OneSeg csrc{c};
-  hooks->before(GL_K_CONV, st);
-  e = launch_conv_one(csrc, c.B, MODE_SIM, st, c.B < num_sms());
-  if (e != cudaSuccess) return e;
-  return hooks->after(GL_K_CONV, st);
+  return launch_conv_single(OneSeg{c}, MODE_SIM, st, hooks);
 }
 
 cudaError_t launch_table(const Seg* d_segs, int nseg, int vec_total, int ray_total, const ConvRun* conv, int nconv,
@@ -2581,27 +2684,28 @@ cudaError_t launch_table(const Seg* d_segs, int nseg, int vec_total, int ray_tot
 // every convolution class launched (an empty class exits at once). Safe to
 // capture into a CUDA graph; conv_smem[c] is the dynamic shared memory of
 // class c and must cover every segment of that class.
-template <int K, int R, int NT, int MINB>
+template <int K, int NT, int MINB>
 static cudaError_t set_devtable_attr(size_t smem) {
-  if (smem > 48 * 1024) {
+  if (smem > DEFAULT_DYN_SMEM) {
     cudaError_t e =
-        cudaFuncSetAttribute(k_conv<K, R, NT, MINB, DevTable>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+        cudaFuncSetAttribute(k_conv<K, NT, MINB, DevTable>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
     if (e != cudaSuccess) return e;
   }
   int resident = 0;   // the occupancy query before any capture
-  return conv_resident<K, R, NT, MINB, DevTable>(smem, &resident);
+  return conv_resident<K, NT, MINB, DevTable>(smem, &resident);
 }
 
 cudaError_t prepare_devtable(const size_t* conv_smem) {
   cudaError_t e;
   (void)fwd_blocks_per_sm();   // the occupancy query before any capture
-  e = conv_smem[0] > CONV_WIDE_MIN_SMEM ? set_devtable_attr<11, 16, 512, 1>(conv_smem[0])
-                                        : set_devtable_attr<11, 16, 256, 3>(conv_smem[0]);
+  e = conv_smem[0] > CONV_WIDE_MIN_SMEM ? set_devtable_attr<11, 512, 1>(conv_smem[0])
+                                        : set_devtable_attr<11, 256, 3>(conv_smem[0]);
   if (e != cudaSuccess) return e;
-  e = conv_smem[1] > CONV_WIDE_MIN_SMEM ? set_devtable_attr<21, 16, 512, 1>(conv_smem[1])
-                                        : set_devtable_attr<21, 16, 256, 1>(conv_smem[1]);
+  e = conv_smem[1] > CONV_WIDE_MIN_SMEM ? set_devtable_attr<21, 512, 1>(conv_smem[1])
+                                        : set_devtable_attr<21, 256, 1>(conv_smem[1]);
   if (e != cudaSuccess) return e;
-  return set_devtable_attr<0, 8, 128, 4>(conv_smem[2]);
+  return conv_smem[2] > CONV_WIDE_MIN_SMEM ? set_devtable_attr<0, 512, 1>(conv_smem[2])
+                                           : set_devtable_attr<0, 256, 2>(conv_smem[2]);
 }
 
 cudaError_t launch_devtable(const TableHdr* d_hdr, const Seg* d_segs, const size_t* conv_smem, cudaStream_t st,

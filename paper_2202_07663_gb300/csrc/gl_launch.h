@@ -35,6 +35,9 @@ constexpr size_t CONV_TWO_BUF_MAX_SMEM = 200 * 1024;
 // it with 512 threads (16 warps) instead of 128 or 256.
 constexpr size_t CONV_WIDE_MIN_SMEM = 100 * 1024;
 
+// Whether a system of this size takes the row-strip form of the 2-D convolution.
+bool conv_rows_fit(int H, int W, int K);
+
 // Whether the convolution of an H x W image, K x K PSF uses the second buffer.
 bool conv_two_buf(int H, int W, int K);
 // Shared memory of the separable convolution (rank-R PSF), whether a system
