@@ -194,6 +194,15 @@ int gl_loglik_grad(gl_system* sys, const float* params, int B, double* loglik_ou
                    double* grad_out, void* stream);
 
 /*
+ * gl_loglik_grad_f32 - gl_loglik_grad (grad_out given) or gl_loglik (NULL) with
+ * log L rounded to float32 [B], for callers that differentiate in float32
+ * (Sec. 2.2): the same numbers as rounding their float64 result, without a
+ * second pass. grad_out [B, 22] stays float64. Device pointers; asynchronous.
+ */
+int gl_loglik_grad_f32(gl_system* sys, const float* params, int B, float* loglik_out, double* grad_out,
+                       void* stream);
+
+/*
  * gl_loglik_grad_host - gl_loglik_grad with HOST buffers: copies params in,
  * computes, copies the results out and synchronises the stream before
  * returning. params/loglik_out/grad_out are host memory (pinned is fastest);
@@ -448,6 +457,16 @@ int gl_hmc_leapfrog_whitened_chain(int B, double* x, double* p, double* z, const
                                    const double* inv_mass, double eps, const double* eps_dev, double kick,
                                    const double* mu, const double* L, const gl_prior_entry* prior, float* theta_out,
                                    void* stream);
+
+/*
+ * gl_scale_rows_f32 - out[b][j] = (float)(scale[b] * rows[b][j]), the product
+ * in FP64: the vector-Jacobian product of a float32 log-likelihood (Sec. 2.2)
+ * from its float64 gradient rows [B, d] and the incoming gradient scale, whose
+ * entry b sits at scale[b * scale_stride] (0 for one value expanded over the
+ * batch). Device pointers; out [B, d] must not alias the inputs; d <= 4096.
+ */
+int gl_scale_rows_f32(int B, int d, const float* scale, size_t scale_stride, const double* rows, float* out,
+                      void* stream);
 
 /*
  * Dense preconditioning (Sec. 2.5: the mass matrix set to the inverse of a

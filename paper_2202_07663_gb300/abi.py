@@ -44,6 +44,7 @@ SIGNATURES = {
     "gl_system_scratch_held": ([_vp], ctypes.c_size_t),
     "gl_loglik": ([_vp, _vp, _i, _vp, _vp, _vp], _i),
     "gl_loglik_grad": ([_vp, _vp, _i, _vp, _vp, _vp, _vp], _i),
+    "gl_loglik_grad_f32": ([_vp, _vp, _i, _vp, _vp, _vp], _i),
     "gl_loglik_grad_host": ([_vp, _vp, _i, _vp, _vp, _vp, _vp], _i),
     "gl_simulate": ([_vp, _vp, _i, _vp, _vp], _i),
     "gl_loglik_grad_grouped": ([_vp, _vp, _vp, _vp, _vp, _vp, _i, _vp], _i),
@@ -61,6 +62,7 @@ SIGNATURES = {
     "gl_hmc_finish": ([_i, _i, _vp, _vp, _vp, _vp, _vp, _vp, _vp, _vp, _d, _vp, _vp, _vp, _vp, _vp, _vp], _i),
     "gl_hmc_chees": ([_i, _i, _vp, _vp, _vp, _vp, _vp, _d, _vp, _vp], _i),
     "gl_hmc_affine": ([_i, _i, _vp, _vp, _vp, _vp, _vp, _vp], _i),
+    "gl_scale_rows_f32": ([_i, _i, _vp, ctypes.c_size_t, _vp, _vp, _vp], _i),
     "gl_hmc_affine_pullback": ([_i, _i, _vp, _vp, _vp, _vp], _i),
     "gl_vi_param_count": ([_i], ctypes.c_size_t),
     "gl_vi_workspace_bytes": ([_i, _i], ctypes.c_size_t),
@@ -126,8 +128,11 @@ def _check(code: int, where: str) -> None:
 
 
 def _stream_ptr(device=None) -> int:
+    """The current stream's handle (without the Stream object of
+    torch.cuda.current_stream: 7 us of a call's host time)."""
     import torch
-    return torch.cuda.current_stream(device).cuda_stream
+    index = device.index if device is not None else None
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device() if index is None else index)
 
 
 def _dptr(t, dtype, shape=None, name="tensor") -> int:
@@ -217,6 +222,10 @@ def gl_hmc_affine(B, d, x, mu, L, z, z32, stream):
 
 def gl_hmc_affine_pullback(B, d, grad_z, L, grad_x, stream):
     _check(lib_handle().gl_hmc_affine_pullback(B, d, grad_z, L, grad_x, stream), "gl_hmc_affine_pullback")
+
+
+def gl_scale_rows_f32(B, d, scale, scale_stride, rows, out, stream):
+    _check(lib_handle().gl_scale_rows_f32(B, d, scale, scale_stride, rows, out, stream), "gl_scale_rows_f32")
 
 
 def gl_profile_enable(on: bool) -> None:
@@ -364,6 +373,17 @@ class GLSystem:
                        _dptr(c2, torch.float64, (B,), "chi2") if c2 is not None else None,
                        _dptr(g, torch.float64, (B, NPARAM), "grad"), _stream_ptr(params.device))
         return (ll, g, c2) if chi2 else (ll, g)
+
+    def loglik_f32(self, params, grad: bool = True):
+        """(log L [B] float32, grad [B, 22] float64 or None): log L rounded
+        to float32 by the kernel that sums it."""
+        import torch
+        p, B = self._params(params)
+        ll = torch.empty(B, dtype=torch.float32, device=params.device)
+        g = torch.empty(B, NPARAM, dtype=torch.float64, device=params.device) if grad else None
+        _check(lib_handle().gl_loglik_grad_f32(self._h, p, B, ll.data_ptr(), g.data_ptr() if grad else None,
+                                               _stream_ptr(params.device)), "gl_loglik_grad_f32")
+        return ll, g
 
     def loglik_grad_profiled(self, params, grad: bool = True, chi2: bool = False):
         """log L profiled over (I_l, I_s): (loglik [B], grad [B, 22] or None,

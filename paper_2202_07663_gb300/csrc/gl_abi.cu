@@ -302,7 +302,7 @@ int check_call(const gl_system* s, const float* params, int B) {
 }
 
 int run_one(gl_system* s, const float* params, int B, double* ll, double* c2, double* grad, float* sim, int mode,
-            cudaStream_t st) {
+            cudaStream_t st, float* ll32 = nullptr) {
   int ntiles, tile_pix;
   long long partial;
   partial_need(s, B, &ntiles, &tile_pix, &partial);
@@ -310,6 +310,7 @@ int run_one(gl_system* s, const float* params, int B, double* ll, double* c2, do
   if (rc != GL_OK) return rc;
   Seg g = make_seg(s, params, B, ntiles, tile_pix);
   g.loglik = ll;
+  g.loglik32 = ll32;
   g.chi2 = c2;
   g.grad = grad;
   g.sim = sim;
@@ -625,6 +626,15 @@ int gl_loglik_grad_profiled(gl_system* s, const float* params, int B, double* lo
   e = gl_internal::launch_zero_amp_grad(B, grad_out, st);
   if (e != cudaSuccess) return cuda_fail(e, "k_zero_amp_grad");
   return GL_OK;
+}
+
+int gl_loglik_grad_f32(gl_system* s, const float* params, int B, float* loglik_out, double* grad_out, void* stream) {
+  int rc = check_call(s, params, B);
+  if (rc != GL_OK) return rc;
+  if (B == 0) return GL_OK;
+  if (!loglik_out) return fail(GL_ERR_INVALID_ARG, "null loglik_out");
+  return run_one(s, params, B, nullptr, nullptr, grad_out, nullptr, grad_out ? gl::MODE_GRAD : gl::MODE_LOGLIK,
+                 static_cast<cudaStream_t>(stream), loglik_out);
 }
 
 int gl_loglik_grad_host(gl_system* s, const float* params, int B, double* loglik_out, double* chi2_out,

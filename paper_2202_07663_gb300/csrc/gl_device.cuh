@@ -28,7 +28,7 @@
 // gradient with respect to e1, e2 in closed form. The sum runs over the
 // coefficients a_1..a_N (per-vector term count N, so all rays of a vector run
 // the same loop), by Horner's rule on G (one complex multiply-add per term)
-// or by the second-order recurrence of epl_fwd_T (two FMAs per term).
+// or by the second-order recurrence of source_position_T (two FMAs per term).
 //
 // The Sersic profile (Eq. Sersic) uses the same quadratic form for its
 // elliptical radius: q x_l^2 + y_l^2 / q = A dx^2 + 2 B dx dy + C dy^2 with
@@ -125,6 +125,7 @@ struct Seg {
   int tile_pix;            // detector pixels per ray tile
   int ray_order;           // 1: the ray kernels take the vectors in VecConst::order (k_order); 0: as given
   double* loglik;          // [B] or null
+  float* loglik32;         // [B] or null: log L rounded to float32
   double* chi2;            // [B] or null
   double* grad;            // [B, 22] or null
   float* sim;              // [B, H, W] or null
@@ -310,10 +311,12 @@ __device__ __forceinline__ T sersic_fwd_T(const RayLight& L, T px, T py) {
 // 1.4e-7), so longer series keep Horner's rule.
 constexpr int RECURRENCE_MAX_PAIRS = 13;
 
-// EPL deflection, generic in the ray type. A ray inside rho < 1e-6 arcsec gets
-// zero deflection (mask), computed without a branch so pairs stay in lockstep.
+// Source-plane position of a ray, generic in the ray type: beta = theta -
+// alpha_EPL - alpha_shear. A ray inside rho < 1e-6 arcsec gets zero EPL
+// deflection (mask), computed without a branch so pairs stay in lockstep.
+// The signs are laid out so that the deflection leaves through the last FMA.
 template <class T>
-__device__ __forceinline__ void epl_fwd_T(const RayC& V, const float4* ser, T x, T y, T& ax, T& ay) {
+__device__ __forceinline__ void source_position_T(const RayC& V, const float4* ser, T x, T y, T& bx, T& by) {
   const T dx = x - sp<T>(V.xc), dy = y - sp<T>(V.yc);
   // w = z - eps conj(z) = (dx - e1 dx - e2 dy, dy + e1 dy - e2 dx)
   const T wr = fmaT(sp<T>(-V.e1), dx, fmaT(sp<T>(-V.e2), dy, dx));
@@ -325,27 +328,27 @@ __device__ __forceinline__ void epl_fwd_T(const RayC& V, const float4* ser, T x,
   // v = w / conj(w) = (1 - 2 wi^2 / |w|^2, 2 wr wi / |w|^2), u = -conj(eps) v
   const T nm = sp<T>(-2.f) * rcpT(w2c) * wi;
   const T vr = fmaT(wi, nm, sp<T>(1.f)), nvi = wr * nm;
-  const T ur = fmaT(sp<T>(-V.e1), vr, sp<T>(V.e2) * nvi);
-  const T ui = fmaT(sp<T>(V.e2), vr, sp<T>(V.e1) * nvi);
-  // F = 1 + sum_n a_n u^n; the two highest terms start the sum (the table is
-  // zero past the term count), then two more per step
-  T hr, hi;
-  const float4 top = ser[V.npairs - 1];
+  const T nur = fmaT(sp<T>(V.e1), vr, sp<T>(-V.e2) * nvi);
+  const T nui = fmaT(sp<T>(-V.e2), vr, sp<T>(-V.e1) * nvi);
+  // -F = -1 - sum_n a_n u^n; the two highest terms start the sum (the table
+  // is zero past the term count), then two more per step
+  T nhr, nhi;
+  const int top = V.npairs - 1;
   if (V.npairs <= RECURRENCE_MAX_PAIRS) {
-    const T ru = ur + ur, nu2 = sp<T>(-V.u2);
-    T c2 = sp<T>(top.y), c1 = fmaT(ru, c2, sp<T>(top.x));
-    for (int m = V.npairs - 2; m >= 0; --m) {
+    const T ru = sp<T>(-2.f) * nur, nu2 = sp<T>(-V.u2);
+    T c2 = sp<T>(ser[top].y), c1 = fmaT(ru, c2, sp<T>(ser[top].x));
+    for (int m = top - 1; m >= 0; --m) {
       const float2 q = *reinterpret_cast<const float2*>(&ser[m]);
       c2 = fmaT(ru, c1, fmaT(nu2, c2, sp<T>(q.y)));
       c1 = fmaT(ru, c2, fmaT(nu2, c1, sp<T>(q.x)));
     }
-    hr = fmaT(ur, c1, fmaT(nu2, c2, sp<T>(1.f)));
-    hi = ui * c1;
+    nhr = fmaT(nur, c1, fmaT(sp<T>(V.u2), c2, sp<T>(-1.f)));
+    nhi = nui * c1;
   } else {
     // G = sum a_{n+1} u^n by Horner (g = a_n + u g), then F = 1 + u G
-    const T nui = -ui;
-    T gr = fmaT(ur, sp<T>(top.y), sp<T>(top.x)), gi = ui * sp<T>(top.y);
-    for (int m = V.npairs - 2; m >= 0; --m) {
+    const T ur = -nur, ui = -nui;
+    T gr = fmaT(ur, sp<T>(ser[top].y), sp<T>(ser[top].x)), gi = ui * sp<T>(ser[top].y);
+    for (int m = top - 1; m >= 0; --m) {
       const float2 q = *reinterpret_cast<const float2*>(&ser[m]);
       const T n1 = fmaT(ur, gr, fmaT(nui, gi, sp<T>(q.y)));
       gi = fmaT(ur, gi, ui * gr);
@@ -353,20 +356,14 @@ __device__ __forceinline__ void epl_fwd_T(const RayC& V, const float4* ser, T x,
       gi = fmaT(ur, gi, ui * n1);
       gr = n0;
     }
-    hr = fmaT(ur, gr, fmaT(nui, gi, sp<T>(1.f)));
-    hi = fmaT(ur, gi, ui * gr);
+    nhr = fmaT(nur, gr, fmaT(ui, gi, sp<T>(-1.f)));
+    nhi = fmaT(nur, gi, nui * gr);
   }
-  ax = S * fmaT(wr, hr, -(wi * hi));
-  ay = S * fmaT(wr, hi, wi * hr);
-}
-
-// Source-plane position of a ray: lens equation with external shear.
-template <class T>
-__device__ __forceinline__ void source_position_T(const RayC& V, const float4* ser, T x, T y, T& bx, T& by) {
-  T ax, ay;
-  epl_fwd_T(V, ser, x, y, ax, ay);
-  bx = x - ax - fmaT(sp<T>(V.g1), x, sp<T>(V.g2) * y);
-  by = y - ay - fmaT(sp<T>(V.g2), x, sp<T>(-V.g1) * y);
+  // shear, then -alpha = -S w F
+  const T x0 = x - fmaT(sp<T>(V.g1), x, sp<T>(V.g2) * y);
+  const T y0 = y - fmaT(sp<T>(V.g2), x, sp<T>(-V.g1) * y);
+  bx = fmaT(S, fmaT(wr, nhr, wi * -nhi), x0);
+  by = fmaT(S, fmaT(wr, nhi, wi * nhr), y0);
 }
 
 template <class T>

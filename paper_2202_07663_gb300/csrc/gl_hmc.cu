@@ -93,6 +93,13 @@ __global__ void k_affine(int B, int d, const double* __restrict__ x, const doubl
   }
 }
 
+// out[b][j] = (float)(scale[b] rows[b][j]), the product in FP64.
+__global__ void k_scale_rows_f32(int n, int d, const float* __restrict__ scale, size_t stride,
+                                 const double* __restrict__ rows, float* __restrict__ out) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
+    out[i] = float(double(scale[size_t(i / d) * stride]) * rows[i]);
+}
+
 __global__ void k_affine_pullback(int B, int d, const double* __restrict__ gz, const double* __restrict__ Lc,
                                   double* __restrict__ gx) {
   extern __shared__ double sL[];
@@ -275,6 +282,20 @@ int gl_hmc_affine(int B, int d, const double* x, const double* mu, const double*
                                                                                            z32_out);
   cudaError_t e = h->after(GL_K_OTHER, st);
   return e == cudaSuccess ? GL_OK : gl_internal::cuda_error(e, "k_affine");
+}
+
+int gl_scale_rows_f32(int B, int d, const float* scale, size_t scale_stride, const double* rows, float* out,
+                      void* stream) {
+  if (B < 0 || d < 1 || d > 4096 || (long long)B * d > 0x7fffffffLL)
+    return gl_internal::set_error(GL_ERR_INVALID_ARG, "bad B or d");
+  if (B == 0) return GL_OK;
+  if (!scale || !rows || !out) return gl_internal::set_error(GL_ERR_INVALID_ARG, "null pointer");
+  gl::Hooks* h = gl_internal::hooks();
+  cudaStream_t st = static_cast<cudaStream_t>(stream);
+  h->before(GL_K_OTHER, st);
+  k_scale_rows_f32<<<grid_for((long long)B * d, 256), 256, 0, st>>>(B * d, d, scale, scale_stride, rows, out);
+  cudaError_t e = h->after(GL_K_OTHER, st);
+  return e == cudaSuccess ? GL_OK : gl_internal::cuda_error(e, "k_scale_rows_f32");
 }
 
 int gl_hmc_affine_pullback(int B, int d, const double* grad_z, const double* L, double* grad_x_out, void* stream) {

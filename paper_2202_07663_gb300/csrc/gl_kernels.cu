@@ -43,6 +43,22 @@ struct OneSeg {
   __device__ __forceinline__ const Seg* conv_seg(int item, int& local) const { local = item; return &s; }
 };
 
+// Index of the last of the n entries of `begin` (ascending, stride ints apart)
+// that is <= item, for a whole warp that asks for the same item: the lanes
+// read the entries side by side instead of one after the other.
+__device__ __forceinline__ int warp_find(const int* begin, int stride, int n, int item) {
+  const int lane = threadIdx.x & 31;
+  int count = 0;
+  for (int i0 = 0; i0 < n; i0 += 32) {
+    const int i = i0 + lane;
+    const bool le = i < n && begin[size_t(i) * stride] <= item;
+    count += __popc(__ballot_sync(0xffffffffu, le));
+  }
+  return count > 0 ? count - 1 : 0;
+}
+constexpr int SEG_INTS = sizeof(Seg) / sizeof(int);
+static_assert(sizeof(Seg) % sizeof(int) == 0, "the segment table is strided in ints");
+
 // Segments in device memory. The convolution kernel of one PSF class sees
 // the contiguous run [conv_first, conv_first + conv_nseg) of the table.
 struct SegTable {
@@ -54,8 +70,7 @@ struct SegTable {
   __device__ __forceinline__ int nconv() const { return conv_total; }
   __device__ __forceinline__ const Seg* conv_seg(int item, int& local) const {
     const Seg* c = segs + conv_first;
-    int lo = 0;
-    for (int i = 1; i < conv_nseg; ++i) lo = (c[i].conv_begin <= item) ? i : lo;
+    const int lo = warp_find(&c->conv_begin, SEG_INTS, conv_nseg, item);
     local = item - c[lo].conv_begin;
     return c + lo;
   }
@@ -66,8 +81,7 @@ struct SegTable {
     return segs + lo;
   }
   __device__ __forceinline__ const Seg* ray_seg(int item, int& local) const {
-    int lo = 0;
-    for (int i = 1; i < nseg; ++i) lo = (segs[i].ray_begin <= item) ? i : lo;
+    const int lo = warp_find(&segs->ray_begin, SEG_INTS, nseg, item);
     local = item - segs[lo].ray_begin;
     return segs + lo;
   }
@@ -90,17 +104,13 @@ struct DevTable {
     return segs + lo;
   }
   __device__ __forceinline__ const Seg* ray_seg(int item, int& local) const {
-    const int n = hdr->nseg;
-    int lo = 0;
-    for (int i = 1; i < n; ++i) lo = (segs[i].ray_begin <= item) ? i : lo;
+    const int lo = warp_find(&segs->ray_begin, SEG_INTS, hdr->nseg, item);
     local = item - segs[lo].ray_begin;
     return segs + lo;
   }
   __device__ __forceinline__ const Seg* conv_seg(int item, int& local) const {
     const Seg* c = segs + hdr->conv_first[cls];
-    const int n = hdr->conv_nseg[cls];
-    int lo = 0;
-    for (int i = 1; i < n; ++i) lo = (c[i].conv_begin <= item) ? i : lo;
+    const int lo = warp_find(&c->conv_begin, SEG_INTS, hdr->conv_nseg[cls], item);
     local = item - c[lo].conv_begin;
     return c + lo;
   }
@@ -145,6 +155,13 @@ __device__ __forceinline__ int setup_vector(const Seg& s, int p) {
 __device__ __forceinline__ void ray_item(const Seg& ss, int local, int& q, int& tile) {
   q = local / ss.ntiles;
   tile = local - q * ss.ntiles;
+}
+
+// Vector b's sums over pixels: L of chi^2 terms and log(2 pi v), C of chi^2.
+__device__ __forceinline__ void store_loglik(const Seg& s, int b, double L, double C) {
+  if (s.loglik) s.loglik[b] = -0.5 * L;
+  if (s.loglik32) s.loglik32[b] = float(-0.5 * L);
+  if (s.chi2) s.chi2[b] = C;
 }
 
 // ------------------------------------------------------------- k_setup ----
@@ -384,11 +401,13 @@ __global__ void k_setup(const __grid_constant__ Src src) {
 // grows like log(tol) / log|eps|, and the key is 204.8 / -log2(|eps|^2)
 // (about four keys per term at tol = 2e-8), capped at NMAX - 1.
 //
-// Two kernels, both before k_setup, using the start of the work buffer
+// One or two kernels before k_setup, using the start of the work buffer
 // (which k_ray_fwd fills only later) as int arrays: key[B], then slot[B],
-// the vector each slot holds. k_keys forms the keys over many blocks (one
-// block reading every vector's row of parameters waits on one SM's
-// scattered loads: 11.8 us at B = 4096). k_order, one block, is a counting
+// the vector each slot holds. Above ORDER_OWN_KEYS vectors k_keys forms the
+// keys over many blocks (one block reading every vector's row of parameters
+// waits on one SM's scattered loads: 11.8 us at B = 4096); up to it, one
+// vector per thread, k_order forms them itself and a launch is saved (B =
+// 300: 21 -> 14 us with its launch between events; the call's launches 7 -> 6). k_order, one block, is a counting
 // sort: each warp counts its vectors per key in a row of its own (shared-
 // memory atomics that never meet another warp's: a batch's keys crowd into
 // a few values, and one counter per key for the whole block would make the
@@ -402,6 +421,7 @@ constexpr int ORDER_THREADS = 1024;
 constexpr int ORDER_WARPS = ORDER_THREADS / 32;
 constexpr int ORDER_UNROLL = 4;         // keys loaded per thread before they are counted
 constexpr int ORDER_PITCH = NMAX + 1;   // per-warp row of counts; the odd pitch spreads the banks
+constexpr int ORDER_OWN_KEYS = ORDER_THREADS;   // batches up to this size form their keys in k_order
 constexpr int ORDER_STAGE = 4096;       // batches up to this size are scattered in shared memory
 static_assert(4 * ORDER_THREADS == ORDER_WARPS * NMAX, "the scan gives each thread four (key, warp) counts");
 
@@ -443,7 +463,7 @@ __global__ void __launch_bounds__(ORDER_THREADS) k_order(const __grid_constant__
   const int chunk = ORDER_UNROLL * ORDER_THREADS;
   const int* keys = order_keys(s);
   int* slots = order_slots(s);
-  const bool staged = B <= ORDER_STAGE;
+  const bool staged = B <= ORDER_STAGE, own = B <= ORDER_OWN_KEYS;
   int* row = cnt + w * ORDER_PITCH;
   for (int i = tid; i < ORDER_WARPS * ORDER_PITCH; i += ORDER_THREADS) cnt[i] = 0;
   __syncthreads();
@@ -451,7 +471,10 @@ __global__ void __launch_bounds__(ORDER_THREADS) k_order(const __grid_constant__
   for (int b0 = tid; b0 - tid < B; b0 += chunk) {   // the same trip count for every thread
     int key[ORDER_UNROLL];
 #pragma unroll
-    for (int u = 0; u < ORDER_UNROLL; ++u) key[u] = order_key_at(keys, b0 + u * ORDER_THREADS, B);
+    for (int u = 0; u < ORDER_UNROLL; ++u) {
+      const int b = b0 + u * ORDER_THREADS;
+      key[u] = own ? (b < B ? order_key(s.params, b) : -1) : order_key_at(keys, b, B);
+    }
 #pragma unroll
     for (int u = 0; u < ORDER_UNROLL; ++u) {
       order_take(row, key[u]);
@@ -710,7 +733,8 @@ __device__ __forceinline__ void light_adj(const RayLight& L, T px, T py, T g, T*
 // 60 x 60, k = 2, B = 4096, 607 -> 459 us; with the signs on the integer pipe
 // and float-stepped grid indices 448, the constants warp-uniform (RayC) and
 // four blocks per SM 406, the series two terms a step and pixels stepped
-// without divisions 396.
+// without divisions 388. The lens light in a loop of its own, so that its
+// eight accumulators are not live with the others: 412.
 //
 // F and the source position stay in Horner's form: next to the source's centre
 // the gradient follows the last bits of the position (a cusp's slope), and
@@ -745,6 +769,7 @@ __device__ __forceinline__ void ray_adj(const RayC& V, const float4* ser, T x, T
   const float4 top = ser[V.npairs - 1];
   T Gr = fmaT(ur, sp<T>(top.y), sp<T>(top.x)), Gi = ui * sp<T>(top.y);
   T c2 = sp<T>(top.w), c1 = fmaT(ru, c2, sp<T>(top.z));
+#pragma unroll 1   // (unrolled by two: 388 -> 396 us; the coefficients as duplicated pairs in shared memory: 403)
   for (int m = V.npairs - 2; m >= 0; --m) {
     const float4 q = ser[m];
     const T n1 = fmaT(ur, Gr, fmaT(nui, Gi, sp<T>(q.y)));
@@ -1013,8 +1038,7 @@ __device__ void conv_vector(const Seg& s, int b, int mode, float* smem, double* 
       L += red2[2 * w];
       C += red2[2 * w + 1];
     }
-    if (s.loglik) s.loglik[b] = -0.5 * L;
-    if (s.chi2) s.chi2[b] = C;
+    store_loglik(s, b, L, C);
   }
   if (!want_grad) return;
   }   // !corr_only
@@ -1074,13 +1098,13 @@ __device__ __forceinline__ float pixel_terms(const Seg& s, int p, float M, float
 // odd side runs in groups of 16 taps and one of K mod 16 (compiled for each
 // remainder), which keeps the loads at one float4 per 32 FMAs or fewer. The
 // column strips that those sides took before read every input value through
-// a scalar load: 61 x 59, K = 13, 200 vectors 131 -> MEAS13 us; 108 x 108,
-// K = 17, one vector 508 -> MEAS17 us (with its row bands).
+// a scalar load: 61 x 59, K = 13, 200 vectors 131 -> 26 us; 108 x 108,
+// K = 17, one vector 508 -> 19.5 us (with its row bands).
 //
 // mirror: the PSF's rows are the same from the top and from the bottom (any
 // profile sampled on a centred grid; gl_system_create checks every value), so
 // the two input rows that meet the same kernel row are added first: (K + 1) / 2
-// rows of FMAs instead of K (K = 21: 100 x 100, B = 512, k_conv 261 -> MEAS21 us).
+// rows of FMAs instead of K (K = 21: 100 x 100, B = 512, k_conv 261 -> 187 us).
 
 // acc[r] += sum_b ker[b] x[r + b], b < G, for the input row at row (and, with
 // two, the one at row2 added to it).
@@ -1222,8 +1246,7 @@ __device__ __forceinline__ void block_loglik(const Seg& s, int b, float ll, floa
       L += red2[2 * w];
       C += red2[2 * w + 1];
     }
-    if (s.loglik) s.loglik[b] = -0.5 * L;
-    if (s.chi2) s.chi2[b] = C;
+    store_loglik(s, b, L, C);
   }
 }
 
@@ -1789,8 +1812,7 @@ __global__ void __launch_bounds__(BAND_THREADS) k_conv_bands(const __grid_consta
       L += bs[0];
       C += bs[1];
     }
-    if (s.loglik) s.loglik[b] = -0.5 * L;
-    if (s.chi2) s.chi2[b] = C;
+    store_loglik(s, b, L, C);
   }
   if (want_grad) {
     // the halo rows of d log L / d M from the bands that own them
@@ -1943,8 +1965,7 @@ __global__ void __launch_bounds__(BAND_THREADS, 2) k_conv_sep_bands(const __grid
         Ls += bs[0];
         Cs += bs[1];
       }
-      if (s.loglik) s.loglik[b] = -0.5 * Ls;
-      if (s.chi2) s.chi2[b] = Cs;
+      store_loglik(s, b, Ls, Cs);
     }
     if (want_grad) {
       // the halo rows of d log L / d M from the bands that own them
@@ -2572,7 +2593,7 @@ static cudaError_t run_rays(const Src& src, int nvec, int nray, bool fwd, bool a
   }
   if (fwd) {
     if (takes_order(src)) {
-      for (int stage = 0; stage < 2; ++stage) {   // k_keys, k_order
+      for (int stage = nvec <= ORDER_OWN_KEYS ? 1 : 0; stage < 2; ++stage) {   // k_keys, k_order
         hooks->before(GL_K_ORDER, st);
         e = launch_order(src, stage, st);
         const cudaError_t h = hooks->after(GL_K_ORDER, st);
@@ -2659,11 +2680,15 @@ cudaError_t launch_basis(const Seg& s, cudaStream_t st, Hooks* hooks) {
   return launch_conv_single(OneSeg{c}, MODE_SIM, st, hooks);
 }
 
+// One block per item, handed out by the hardware as SMs free up: the items of
+// a mixed table differ in cost, and a persistent grid's static split left the
+// SMs with the large systems' items working alone (four systems of 40 x 40 to
+// 80 x 80: 429 -> 385 us a call).
 cudaError_t launch_table(const Seg* d_segs, int nseg, int vec_total, int ray_total, const ConvRun* conv, int nconv,
                          int mode, cudaStream_t st, Hooks* hooks) {
   if (vec_total <= 0) return cudaSuccess;
   SegTable src{d_segs, nseg, vec_total, ray_total, 0, nseg, vec_total};
-  cudaError_t e = run_rays(src, vec_total, ray_total, true, false, st, hooks, true);
+  cudaError_t e = run_rays(src, vec_total, ray_total, true, false, st, hooks, false);
   if (e != cudaSuccess) return e;
   for (int i = 0; i < nconv; ++i) {
     SegTable cs = src;
@@ -2671,13 +2696,13 @@ cudaError_t launch_table(const Seg* d_segs, int nseg, int vec_total, int ray_tot
     cs.conv_nseg = conv[i].nseg;
     cs.conv_total = conv[i].nitems;
     hooks->before(GL_K_CONV, st);
-    e = launch_conv_class(conv[i].cls, cs, conv[i].nitems, conv[i].smem, mode, st, true,
+    e = launch_conv_class(conv[i].cls, cs, conv[i].nitems, conv[i].smem, mode, st, false,
                           conv[i].smem > CONV_WIDE_MIN_SMEM);
     if (e != cudaSuccess) return e;
     if ((e = hooks->after(GL_K_CONV, st)) != cudaSuccess) return e;
   }
   if (mode != MODE_GRAD) return cudaSuccess;
-  return run_rays(src, vec_total, ray_total, false, true, st, hooks, true);
+  return run_rays(src, vec_total, ray_total, false, true, st, hooks, false);
 }
 
 // Grouped launch whose counts live in device memory: fixed persistent grids,

@@ -1,0 +1,70 @@
+"""The fused backward of the autograd log-likelihood (gl_scale_rows_f32)
+against the torch expression it stands for, and the cases that must keep that
+expression: gradients of gradients, batched gradients, float64 parameters."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+import oracle  # noqa: E402
+from paper_2202_07663_gb300 import inputs  # noqa: E402
+from gpu_common import make_system  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def setup():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2202_07663_gb300 import abi, build, hmc
+    build.build()
+    oracle.build()
+    spec = inputs.SystemSpec(20, 23, 1, 5)
+    truth, image, psf = make_system(spec, 31)
+    s = abi.GLSystem(image, psf, spec.pixel_scale, spec.k, spec.gain_exposure, sigma_bkg=spec.sigma_bkg)
+    p = inputs.draw_perturbed(np.random.default_rng(3), truth, 37).astype(np.float32)
+    return hmc, s, torch.from_numpy(p).cuda()
+
+
+@pytest.mark.parametrize("B", [1, 2, 37])
+def test_fused_backward_equals_the_torch_expression(setup, B):
+    hmc, s, p0 = setup
+    p = p0[:B].clone().requires_grad_()
+    g = s.loglik_grad(p0[:B].contiguous())[1]
+    w = torch.randn(2 * B, device="cuda")
+    for make in (lambda ll: ll.sum(), lambda ll: (ll * w[:B]).sum(), lambda ll: (ll * w[::2]).sum(),
+                 lambda ll: ll.mean()):
+        ll = hmc.loglik(p, s)
+        (go,) = torch.autograd.grad(make(ll), ll, retain_graph=True)
+        (out,) = torch.autograd.grad(make(ll), p)
+        assert out.dtype == torch.float32
+        assert torch.equal(out, (go.to(torch.float64)[:, None] * g).to(torch.float32))
+    # a strided incoming gradient
+    ll = hmc.loglik(p, s)
+    (out,) = torch.autograd.grad(ll, p, grad_outputs=w[::2])
+    assert torch.equal(out, (w[::2].to(torch.float64)[:, None] * g).to(torch.float32))
+
+
+def test_other_uses_keep_the_torch_expression(setup):
+    hmc, s, p0 = setup
+    g = s.loglik_grad(p0)[1]
+    # the product's own derivative with respect to the incoming gradient
+    p = p0.clone().requires_grad_()
+    w = torch.randn(len(p0), device="cuda", requires_grad=True)
+    (out,) = torch.autograd.grad(hmc.loglik(p, s), p, grad_outputs=w, create_graph=True)
+    (dw,) = torch.autograd.grad(out.sum(), w)
+    np.testing.assert_allclose(dw.cpu().numpy(), g.sum(1).cpu().numpy(), rtol=1e-5, atol=1e-5 * float(g.abs().max()))
+    # a batch of incoming gradients
+    W = torch.randn(3, len(p0), device="cuda")
+    (out,) = torch.autograd.grad(hmc.loglik(p, s), p, grad_outputs=W, is_grads_batched=True)
+    assert torch.equal(out, (W.to(torch.float64)[:, :, None] * g).to(torch.float32))
+    # float64 parameters
+    q = p0.double().requires_grad_()
+    (out,) = torch.autograd.grad(hmc.loglik(q, s).sum(), q)
+    assert out.dtype == torch.float64 and torch.equal(out, g)
+    # a hook that holds the saved gradient on the host and brings it back
+    with torch.autograd.graph.save_on_cpu():
+        ll = hmc.loglik(p, s)
+    (out,) = torch.autograd.grad(ll.sum(), p)
+    assert torch.equal(out, g.to(torch.float32))
