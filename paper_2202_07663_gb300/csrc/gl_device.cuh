@@ -27,8 +27,7 @@
 // (e1, e2) through e = 0, needs no atan2 and no rotation, and gives the
 // gradient with respect to e1, e2 in closed form. The sum runs over the
 // coefficients a_1..a_N (per-vector term count N, so all rays of a vector run
-// the same loop), by Horner's rule on G (one complex multiply-add per term)
-// or by the second-order recurrence of source_position_T (two FMAs per term).
+// the same loop), by Horner's rule on G: one complex multiply-add per term.
 //
 // The Sersic profile (Eq. Sersic) uses the same quadratic form for its
 // elliptical radius: q x_l^2 + y_l^2 / q = A dx^2 + 2 B dx dy + C dy^2 with
@@ -50,6 +49,7 @@
 #pragma once
 
 #include <cstdint>
+#include <type_traits>
 
 namespace gl {
 
@@ -226,10 +226,11 @@ __device__ __forceinline__ float rcpT(float a) { return rcp(a); }
 __device__ __forceinline__ F2 rcpT(F2 a) { return {make_float2(rcp(a.v.x), rcp(a.v.y))}; }
 __device__ __forceinline__ float maxT(float a, float b) { return fmaxf(a, b); }
 __device__ __forceinline__ F2 maxT(F2 a, F2 b) { return {make_float2(fmaxf(a.v.x, b.v.x), fmaxf(a.v.y, b.v.y))}; }
-// 1 where a >= b, else 0
-__device__ __forceinline__ float geT(float a, float b) { return a >= b ? 1.f : 0.f; }
-__device__ __forceinline__ F2 geT(F2 a, F2 b) {
-  return {make_float2(a.v.x >= b.v.x ? 1.f : 0.f, a.v.y >= b.v.y ? 1.f : 0.f)};
+// v where a >= b, else 0, by selection (a 0/1 factor would be one more
+// instruction of the FP32 pipe)
+__device__ __forceinline__ float where_ge(float a, float b, float v) { return a >= b ? v : 0.f; }
+__device__ __forceinline__ F2 where_ge(F2 a, F2 b, F2 v) {
+  return {make_float2(a.v.x >= b.v.x ? v.v.x : 0.f, a.v.y >= b.v.y ? v.v.y : 0.f)};
 }
 
 // log2 without the bias of lg2.approx. lg2.approx.ftz measured on GB300
@@ -265,8 +266,7 @@ __device__ __forceinline__ F2 grid_coord2(F2 n, float hh, float hl) { return fma
 // that it can hold them in uniform registers: copied from shared memory into
 // ordinary ones they took 31 registers of every thread, and with the 24 packed
 // accumulators the adjoint then fitted three blocks per SM with spills
-// (k_ray_adj at 60 x 60, k = 2, B = 4096: 448.5 -> 428 us at three blocks, and
-// 406 us at the four that fit with them).
+// (k_ray_adj at 60 x 60, k = 2, B = 4096, three blocks per SM: 448.5 -> 428 us).
 struct RayLight {
   float A, B2, C, x, y, c1, r2min, k1, I0;
 };
@@ -296,78 +296,93 @@ __device__ __forceinline__ RayC ray_consts(const VecConst& v) {
 template <class T>
 __device__ __forceinline__ T sersic_fwd_T(const RayLight& L, T px, T py) {
   const T dx = px - sp<T>(L.x), dy = py - sp<T>(L.y);
-  T r2 = fmaT(fmaT(sp<T>(L.A), dx, sp<T>(L.B2) * dy), dx, sp<T>(L.C) * dy * dy);
+  T r2 = fmaT(sp<T>(L.A) * dx, dx, fmaT(sp<T>(L.B2) * dx, dy, sp<T>(L.C) * dy * dy));
   r2 = maxT(r2, sp<T>(L.r2min));
   const T s = ex2T(sp<T>(L.c1) * lg2cT(r2));
   return sp<T>(L.I0) * ex2T(fmaT(sp<T>(-L.k1), s, sp<T>(L.k1)));
 }
 
-// Series of at most 26 terms (|eps| up to about 0.5) are summed by
-// the second-order recurrence for a real polynomial at a complex point
-// (Knuth, TAOCP 4.6.4; |u|^2 = |eps|^2 for every ray): two FMAs a term
-// instead of Horner's four. Its error against 64 bits over |u| = f is
-// Horner's at f <= 0.5 (rms 3.2e-8, max 1.0e-7 for both), above it grows with
-// 1 / (1 - f)^2 (f = 0.7: max 2.4e-7 against 1.1e-7; f = 0.85: 1.0e-6 against
-// 1.4e-7), so longer series keep Horner's rule.
-constexpr int RECURRENCE_MAX_PAIRS = 13;
+// The series table as the ray loops read it. NP > 0: exactly NP pairs of
+// terms, held warp-uniform, so that the sum is straight-line code that the
+// compiler can interleave with the ray's other chains (the lens light's
+// special functions above all); NP == 0: any length, from shared memory.
+// ADJ: with the derivatives b_n. Against the loop for every length, 60 x 60,
+// k = 2, B = 4096: k_ray_fwd 232 -> 197 us, k_ray_adj 388 -> 378 us (367 at three
+// blocks per SM).
+constexpr int SERIES_UNROLL = 6;   // longest compiled length in pairs (12 terms: |eps| up to about 0.25)
+template <int NP, bool ADJ>
+struct Series {
+  float a[2 * NP], b[ADJ ? 2 * NP : 1];
+  __device__ __forceinline__ Series(const float4* ser) {
+#pragma unroll
+    for (int m = 0; m < NP; ++m) {
+      const float4 q = ser[m];
+      a[2 * m] = warp_uniform(q.x);
+      a[2 * m + 1] = warp_uniform(q.y);
+      if constexpr (ADJ) {
+        b[2 * m] = warp_uniform(q.z);
+        b[2 * m + 1] = warp_uniform(q.w);
+      }
+    }
+  }
+  __device__ __forceinline__ float4 pair(int m) const { return {a[2 * m], a[2 * m + 1], ADJ ? b[2 * m] : 0.f, ADJ ? b[2 * m + 1] : 0.f}; }
+};
+template <bool ADJ>
+struct Series<0, ADJ> {
+  const float4* ser;
+  __device__ __forceinline__ Series(const float4* s) : ser(s) {}
+  __device__ __forceinline__ float4 pair(int m) const { return ser[m]; }
+};
 
 // Source-plane position of a ray, generic in the ray type: beta = theta -
 // alpha_EPL - alpha_shear. A ray inside rho < 1e-6 arcsec gets zero EPL
 // deflection (mask), computed without a branch so pairs stay in lockstep.
-// The signs are laid out so that the deflection leaves through the last FMA.
-template <class T>
-__device__ __forceinline__ void source_position_T(const RayC& V, const float4* ser, T x, T y, T& bx, T& by) {
+// G = sum_{n<N} a_{n+1} u^n by Horner's rule; the two highest terms start the
+// sum (the table is zero past the term count), then two more per step. The
+// adjoint evaluates the same expressions, so both kernels see the same
+// positions, and next to a light's centre both the image and the gradient
+// follow their last bits. (The sum by a second-order recurrence, two FMAs a
+// term instead of four, Knuth TAOCP 4.6.4, is as accurate up to |eps| = 0.5 and
+// took k_ray_fwd at 60 x 60, B = 4096 from 197 to 162 us, but near a mode it
+// moved the gradients of a batch by up to 3e-5 of their norm; not kept.)
+template <int NP, bool ADJ, class T>
+__device__ __forceinline__ void source_position_T(const RayC& V, const Series<NP, ADJ>& ser, T x, T y, T& bx, T& by) {
   const T dx = x - sp<T>(V.xc), dy = y - sp<T>(V.yc);
   // w = z - eps conj(z) = (dx - e1 dx - e2 dy, dy + e1 dy - e2 dx)
   const T wr = fmaT(sp<T>(-V.e1), dx, fmaT(sp<T>(-V.e2), dy, dx));
   const T wi = fmaT(sp<T>(V.e1), dy, fmaT(sp<T>(-V.e2), dx, dy));
   const T w2 = fmaT(wr, wr, wi * wi);
-  const T keep = geT(w2, sp<T>(V.w2min));
-  const T w2c = maxT(w2, sp<T>(V.w2min));   // > 0; where it clamps, keep = 0 zeroes the deflection
-  const T S = keep * ex2T(fmaT(sp<T>(V.t), fmaT(sp<T>(-0.5f), lg2T(w2c), sp<T>(V.lc)), sp<T>(V.tlc_lo)));
-  // v = w / conj(w) = (1 - 2 wi^2 / |w|^2, 2 wr wi / |w|^2), u = -conj(eps) v
-  const T nm = sp<T>(-2.f) * rcpT(w2c) * wi;
-  const T vr = fmaT(wi, nm, sp<T>(1.f)), nvi = wr * nm;
-  const T nur = fmaT(sp<T>(V.e1), vr, sp<T>(-V.e2) * nvi);
-  const T nui = fmaT(sp<T>(-V.e2), vr, sp<T>(-V.e1) * nvi);
-  // -F = -1 - sum_n a_n u^n; the two highest terms start the sum (the table
-  // is zero past the term count), then two more per step
-  T nhr, nhi;
-  const int top = V.npairs - 1;
-  if (V.npairs <= RECURRENCE_MAX_PAIRS) {
-    const T ru = sp<T>(-2.f) * nur, nu2 = sp<T>(-V.u2);
-    T c2 = sp<T>(ser[top].y), c1 = fmaT(ru, c2, sp<T>(ser[top].x));
-    for (int m = top - 1; m >= 0; --m) {
-      const float2 q = *reinterpret_cast<const float2*>(&ser[m]);
-      c2 = fmaT(ru, c1, fmaT(nu2, c2, sp<T>(q.y)));
-      c1 = fmaT(ru, c2, fmaT(nu2, c1, sp<T>(q.x)));
-    }
-    nhr = fmaT(nur, c1, fmaT(sp<T>(V.u2), c2, sp<T>(-1.f)));
-    nhi = nui * c1;
-  } else {
-    // G = sum a_{n+1} u^n by Horner (g = a_n + u g), then F = 1 + u G
-    const T ur = -nur, ui = -nui;
-    T gr = fmaT(ur, sp<T>(ser[top].y), sp<T>(ser[top].x)), gi = ui * sp<T>(ser[top].y);
-    for (int m = top - 1; m >= 0; --m) {
-      const float2 q = *reinterpret_cast<const float2*>(&ser[m]);
-      const T n1 = fmaT(ur, gr, fmaT(nui, gi, sp<T>(q.y)));
-      gi = fmaT(ur, gi, ui * gr);
-      const T n0 = fmaT(ur, n1, fmaT(nui, gi, sp<T>(q.x)));
-      gi = fmaT(ur, gi, ui * n1);
-      gr = n0;
-    }
-    nhr = fmaT(nur, gr, fmaT(ui, gi, sp<T>(-1.f)));
-    nhi = fmaT(nur, gi, nui * gr);
+  const T w2c = maxT(w2, sp<T>(V.w2min));   // > 0; where it clamps, S = 0 zeroes the deflection
+  const T S = where_ge(w2, sp<T>(V.w2min),
+                       ex2T(fmaT(sp<T>(V.t), fmaT(sp<T>(-0.5f), lg2T(w2c), sp<T>(V.lc)), sp<T>(V.tlc_lo))));
+  const T iw2 = rcpT(w2c);
+  const T nwi = -wi;
+  const T vr = fmaT(wr, wr, nwi * wi) * iw2;
+  const T vh = wr * wi * iw2;   // Im v / 2 (twice it goes into the constants: the same bits)
+  const T ur = fmaT(sp<T>(-V.e1), vr, sp<T>(-2.f * V.e2) * vh);
+  const T ui = fmaT(sp<T>(V.e2), vr, sp<T>(-2.f * V.e1) * vh);
+  const T nui = -ui;            // packed FMAs take no negated operands
+  const int np = NP > 0 ? NP : V.npairs;
+  const float4 top = ser.pair(np - 1);
+  T gr = fmaT(ur, sp<T>(top.y), sp<T>(top.x)), gi = ui * sp<T>(top.y);
+#pragma unroll (NP > 0 ? SERIES_UNROLL : 2)
+  for (int m = np - 2; m >= 0; --m) {
+    const float4 q = ser.pair(m);
+    const T n1 = fmaT(ur, gr, fmaT(nui, gi, sp<T>(q.y)));
+    gi = fmaT(ur, gi, ui * gr);
+    gr = fmaT(ur, n1, fmaT(nui, gi, sp<T>(q.x)));
+    gi = fmaT(ur, gi, ui * n1);
   }
-  // shear, then -alpha = -S w F
-  const T x0 = x - fmaT(sp<T>(V.g1), x, sp<T>(V.g2) * y);
-  const T y0 = y - fmaT(sp<T>(V.g2), x, sp<T>(-V.g1) * y);
-  bx = fmaT(S, fmaT(wr, nhr, wi * -nhi), x0);
-  by = fmaT(S, fmaT(wr, nhi, wi * nhr), y0);
+  const T hr = fmaT(ur, gr, fmaT(nui, gi, sp<T>(1.f)));   // F = 1 + u G
+  const T hi = fmaT(ur, gi, ui * gr);
+  const T ax = S * fmaT(wr, hr, nwi * hi);
+  const T ay = S * fmaT(wr, hi, wi * hr);
+  bx = x - ax - fmaT(sp<T>(V.g1), x, sp<T>(V.g2) * y);
+  by = y - ay - fmaT(sp<T>(V.g2), x, sp<T>(-V.g1) * y);
 }
 
-template <class T>
-__device__ __forceinline__ T ray_intensity_T(const RayC& V, const float4* ser, T x, T y) {
+template <int NP, bool ADJ, class T>
+__device__ __forceinline__ T ray_intensity_T(const RayC& V, const Series<NP, ADJ>& ser, T x, T y) {
   T bx, by;
   source_position_T(V, ser, x, y, bx, by);
   return sersic_fwd_T(V.light[1], bx, by) + sersic_fwd_T(V.light[0], x, y);
@@ -388,5 +403,21 @@ struct PixelStep {
     }
   }
 };
+
+// Runs f(integral_constant NP) for the vector's series length: its number of
+// pairs up to SERIES_UNROLL, else 0. Block-uniform.
+template <class F>
+__device__ __forceinline__ void with_series(int npairs, F&& f) {
+  switch (npairs) {
+    case 1: f(std::integral_constant<int, 1>{}); break;
+    case 2: f(std::integral_constant<int, 2>{}); break;
+    case 3: f(std::integral_constant<int, 3>{}); break;
+    case 4: f(std::integral_constant<int, 4>{}); break;
+    case 5: f(std::integral_constant<int, 5>{}); break;
+    case 6: f(std::integral_constant<int, 6>{}); break;
+    default: f(std::integral_constant<int, 0>{}); break;
+  }
+}
+static_assert(SERIES_UNROLL == 6, "with_series lists the compiled lengths");
 
 }  // namespace gl

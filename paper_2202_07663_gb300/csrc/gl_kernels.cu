@@ -543,14 +543,15 @@ __global__ void __launch_bounds__(ORDER_THREADS) k_order(const __grid_constant__
 
 // ----------------------------------------------------------- k_ray_fwd ----
 
-// Block size and resident blocks per SM of the forward kernel. It is bound by
-// issue slots and the FP32 pipe together (65% and 62% busy). At 60 x 60, k = 2,
-// B = 4096, blocks of 128 threads: four per SM (105 registers) 211 us, five
-// (95) 198, six (80, 52 bytes of spills) 201, seven 205; 244 us before the
-// series went from Horner's rule to the second-order recurrence, the
-// constants became warp-uniform and the divisions left the pixel loop.
+// Block size and resident blocks per SM of the forward kernel, bound by the
+// FP32 pipe and the latency between its special functions. 60 x 60, k = 2, B =
+// 4096: 244 us with the constants copied per thread, a division per pixel and
+// the series in a loop; now 197. By blocks of 128 threads per SM (before the
+// last two operations of the Sersic radius): 4 (110 registers) 205, 5 (91) 197,
+// 6 (79) 192.5, 7 (72, 4 bytes of spills) 192 us; 200 x 200, k = 4, B = 1024 2011,
+// 1930, 1891, 1888 us.
 constexpr int FWD_THREADS = 128;
-constexpr int FWD_BLOCKS_PER_SM = 5;
+constexpr int FWD_BLOCKS_PER_SM = 7;
 
 template <class Src>
 __global__ void __launch_bounds__(FWD_THREADS, FWD_BLOCKS_PER_SM) k_ray_fwd(const __grid_constant__ Src src) {
@@ -574,35 +575,38 @@ __global__ void __launch_bounds__(FWD_THREADS, FWD_BLOCKS_PER_SM) k_ray_fwd(cons
     const bool valid = sv.nterms >= 0;
     const RayC rc = ray_consts(sv);
     float* out = ss.work + size_t(b) * HW;
-    // two pixels per thread and step (p and p + blockDim), their rays paired in f32x2
-    const int stride = blockDim.x;
-    const PixelStep step(2 * stride, W);
-    int ip = (p0 + int(threadIdx.x)) / W, jp = p0 + int(threadIdx.x) - ip * W;
-    int iq = (p0 + int(threadIdx.x) + stride) / W, jq = p0 + int(threadIdx.x) + stride - iq * W;
-    for (int p = p0 + threadIdx.x; p < p1; p += 2 * stride, step.advance(ip, jp, W), step.advance(iq, jq, W)) {
-      const int q = p + stride;   // past the tile: its rays are computed and not stored
-      const bool has_q = q < p1;
-      F2 acc = sp<F2>(0.f);
-      if (valid) {
-        // grid indices of the pixels' first subpixels; a subpixel step adds 2
-        const F2 ny0 = {make_float2(float(2 * ip * k + ss.ny0), float(2 * iq * k + ss.ny0))};
-        const F2 nx0 = {make_float2(float(2 * jp * k + ss.nx0), float(2 * jq * k + ss.nx0))};
-        F2 ny = ny0;
-        for (int a = 0; a < k; ++a, ny = ny + sp<F2>(2.f)) {
-          const F2 y = grid_coord2(ny, ss.hh, ss.hl);
-          F2 nx = nx0;
-          for (int c = 0; c < k; ++c, nx = nx + sp<F2>(2.f)) {
-            const F2 x = grid_coord2(nx, ss.hh, ss.hl);
-            acc = acc + ray_intensity_T(rc, sv.ser, x, y);
+    with_series(valid ? rc.npairs : 0, [&](auto np) {
+      const Series<decltype(np)::value, false> ser(sv.ser);
+      // two pixels per thread and step (p and p + blockDim), their rays paired in f32x2
+      const int stride = blockDim.x;
+      const PixelStep step(2 * stride, W);
+      int ip = (p0 + int(threadIdx.x)) / W, jp = p0 + int(threadIdx.x) - ip * W;
+      int iq = (p0 + int(threadIdx.x) + stride) / W, jq = p0 + int(threadIdx.x) + stride - iq * W;
+      for (int p = p0 + threadIdx.x; p < p1; p += 2 * stride, step.advance(ip, jp, W), step.advance(iq, jq, W)) {
+        const int q = p + stride;   // past the tile: its rays are computed and not stored
+        const bool has_q = q < p1;
+        F2 acc = sp<F2>(0.f);
+        if (valid) {
+          // grid indices of the pixels' first subpixels; a subpixel step adds 2
+          const F2 ny0 = {make_float2(float(2 * ip * k + ss.ny0), float(2 * iq * k + ss.ny0))};
+          const F2 nx0 = {make_float2(float(2 * jp * k + ss.nx0), float(2 * jq * k + ss.nx0))};
+          F2 ny = ny0;
+          for (int a = 0; a < k; ++a, ny = ny + sp<F2>(2.f)) {
+            const F2 y = grid_coord2(ny, ss.hh, ss.hl);
+            F2 nx = nx0;
+            for (int c = 0; c < k; ++c, nx = nx + sp<F2>(2.f)) {
+              const F2 x = grid_coord2(nx, ss.hh, ss.hl);
+              acc = acc + ray_intensity_T(rc, ser, x, y);
+            }
           }
+          acc = acc * sp<F2>(inv_k2);
+        } else {
+          acc = sp<F2>(__int_as_float(0x7fc00000));
         }
-        acc = acc * sp<F2>(inv_k2);
-      } else {
-        acc = sp<F2>(__int_as_float(0x7fc00000));
+        out[p] = acc.v.x;
+        if (has_q) out[q] = acc.v.y;
       }
-      out[p] = acc.v.x;
-      if (has_q) out[q] = acc.v.y;
-    }
+    });
     __syncthreads();
   }
 }
@@ -636,41 +640,44 @@ __global__ void __launch_bounds__(FWD_THREADS, FWD_BLOCKS_PER_SM) k_ray_fwd_basi
     const bool valid = sv.nterms >= 0;
     float* out_l = ss.work + size_t(2 * b) * HW;
     float* out_s = out_l + HW;
-    const int stride = blockDim.x;
-    const PixelStep step(2 * stride, W);
-    int ip = (p0 + int(threadIdx.x)) / W, jp = p0 + int(threadIdx.x) - ip * W;
-    int iq = (p0 + int(threadIdx.x) + stride) / W, jq = p0 + int(threadIdx.x) + stride - iq * W;
-    for (int p = p0 + threadIdx.x; p < p1; p += 2 * stride, step.advance(ip, jp, W), step.advance(iq, jq, W)) {
-      const int q = p + stride;   // past the tile: its rays are computed and not stored
-      const bool has_q = q < p1;
-      F2 acc_l = sp<F2>(0.f), acc_s = sp<F2>(0.f);
-      if (valid) {
-        const F2 ny0 = {make_float2(float(2 * ip * k + ss.ny0), float(2 * iq * k + ss.ny0))};
-        const F2 nx0 = {make_float2(float(2 * jp * k + ss.nx0), float(2 * jq * k + ss.nx0))};
-        F2 ny = ny0;
-        for (int a = 0; a < k; ++a, ny = ny + sp<F2>(2.f)) {
-          const F2 y = grid_coord2(ny, ss.hh, ss.hl);
-          F2 nx = nx0;
-          for (int c = 0; c < k; ++c, nx = nx + sp<F2>(2.f)) {
-            const F2 x = grid_coord2(nx, ss.hh, ss.hl);
-            F2 bx, by;
-            source_position_T(rc, sv.ser, x, y, bx, by);
-            acc_s = acc_s + sersic_fwd_T(rc.light[1], bx, by);
-            acc_l = acc_l + sersic_fwd_T(rc.light[0], x, y);
+    with_series(valid ? rc.npairs : 0, [&](auto np) {
+      const Series<decltype(np)::value, false> ser(sv.ser);
+      const int stride = blockDim.x;
+      const PixelStep step(2 * stride, W);
+      int ip = (p0 + int(threadIdx.x)) / W, jp = p0 + int(threadIdx.x) - ip * W;
+      int iq = (p0 + int(threadIdx.x) + stride) / W, jq = p0 + int(threadIdx.x) + stride - iq * W;
+      for (int p = p0 + threadIdx.x; p < p1; p += 2 * stride, step.advance(ip, jp, W), step.advance(iq, jq, W)) {
+        const int q = p + stride;   // past the tile: its rays are computed and not stored
+        const bool has_q = q < p1;
+        F2 acc_l = sp<F2>(0.f), acc_s = sp<F2>(0.f);
+        if (valid) {
+          const F2 ny0 = {make_float2(float(2 * ip * k + ss.ny0), float(2 * iq * k + ss.ny0))};
+          const F2 nx0 = {make_float2(float(2 * jp * k + ss.nx0), float(2 * jq * k + ss.nx0))};
+          F2 ny = ny0;
+          for (int a = 0; a < k; ++a, ny = ny + sp<F2>(2.f)) {
+            const F2 y = grid_coord2(ny, ss.hh, ss.hl);
+            F2 nx = nx0;
+            for (int c = 0; c < k; ++c, nx = nx + sp<F2>(2.f)) {
+              const F2 x = grid_coord2(nx, ss.hh, ss.hl);
+              F2 bx, by;
+              source_position_T(rc, ser, x, y, bx, by);
+              acc_s = acc_s + sersic_fwd_T(rc.light[1], bx, by);
+              acc_l = acc_l + sersic_fwd_T(rc.light[0], x, y);
+            }
           }
+          acc_l = acc_l * sp<F2>(inv_k2);
+          acc_s = acc_s * sp<F2>(inv_k2);
+        } else {
+          acc_l = acc_s = sp<F2>(__int_as_float(0x7fc00000));
         }
-        acc_l = acc_l * sp<F2>(inv_k2);
-        acc_s = acc_s * sp<F2>(inv_k2);
-      } else {
-        acc_l = acc_s = sp<F2>(__int_as_float(0x7fc00000));
+        out_l[p] = acc_l.v.x;
+        out_s[p] = acc_s.v.x;
+        if (has_q) {
+          out_l[q] = acc_l.v.y;
+          out_s[q] = acc_s.v.y;
+        }
       }
-      out_l[p] = acc_l.v.x;
-      out_s[p] = acc_s.v.x;
-      if (has_q) {
-        out_l[q] = acc_l.v.y;
-        out_s[q] = acc_s.v.y;
-      }
-    }
+    });
     __syncthreads();
   }
 }
@@ -686,23 +693,29 @@ __global__ void __launch_bounds__(FWD_THREADS, FWD_BLOCKS_PER_SM) k_ray_fwd_basi
 //   acc[7] g e
 // The profile's eight derivatives are linear in these with coefficients that
 // every ray of a vector shares (A, B, C and their derivatives in e1, e2), so
-// k_final forms them once per vector instead of each ray. Returns gq dx and
-// gq dy: (A qx + B qy, B qx + C qy) is the ray's position derivative over
-// -(b_n / n) I0. Generic in the ray type (float or a packed pair).
-template <class T>
-__device__ __forceinline__ void light_adj(const RayLight& L, T px, T py, T g, T* acc, T& qx, T& qy) {
+// k_final forms them once per vector instead of each ray. With POS also
+// returns Gx = gq (A dx + B dy), Gy = gq (B dx + C dy) (B = B2 / 2): the ray's
+// position derivative over -(b_n / n) I0. Generic in the ray type (float or a
+// packed pair).
+template <bool POS, class T>
+__device__ __forceinline__ void light_adj(const RayLight& L, T px, T py, T g, T* acc, T& Gx, T& Gy) {
   const T dx = px - sp<T>(L.x), dy = py - sp<T>(L.y);
-  const T m = fmaT(sp<T>(L.B2), dy, sp<T>(L.A) * dx);
-  const T r2raw = fmaT(m, dx, sp<T>(L.C) * dy * dy);
-  const T keep = geT(r2raw, sp<T>(L.r2min));       // 0 where the radius is floored
+  T hx, hy, r2raw;
+  if constexpr (POS) {
+    const float Bh = 0.5f * L.B2;
+    hx = fmaT(sp<T>(L.A), dx, sp<T>(Bh) * dy);
+    hy = fmaT(sp<T>(Bh), dx, sp<T>(L.C) * dy);
+    r2raw = fmaT(hx, dx, hy * dy);
+  } else {
+    r2raw = fmaT(fmaT(sp<T>(L.A), dx, sp<T>(L.B2) * dy), dx, sp<T>(L.C) * dy * dy);
+  }
   const T r2 = maxT(r2raw, sp<T>(L.r2min));
   const T ls = sp<T>(L.c1) * lg2T(r2);
   const T s = ex2T(ls);
   const T ge = g * ex2T(fmaT(sp<T>(-L.k1), s, sp<T>(L.k1)));
   const T hs = ge * s;
-  const T gq = keep * hs * rcpT(r2);
-  qx = gq * dx;
-  qy = gq * dy;
+  const T gq = hs * where_ge(r2raw, sp<T>(L.r2min), rcpT(r2));   // 0 where the radius is floored
+  const T qx = gq * dx, qy = gq * dy;
   acc[0] = acc[0] + hs;
   acc[1] = fmaT(hs, ls, acc[1]);
   acc[2] = acc[2] + qx;
@@ -711,6 +724,10 @@ __device__ __forceinline__ void light_adj(const RayLight& L, T px, T py, T g, T*
   acc[5] = fmaT(qx, dy, acc[5]);
   acc[6] = fmaT(qy, dy, acc[6]);
   acc[7] = acc[7] + ge;
+  if constexpr (POS) {
+    Gx = gq * hx;
+    Gy = gq * hy;
+  }
 }
 
 // One ray (or a packed pair): adds its share of the 24 accumulators. The mass
@@ -733,7 +750,7 @@ __device__ __forceinline__ void light_adj(const RayLight& L, T px, T py, T g, T*
 // 60 x 60, k = 2, B = 4096, 607 -> 459 us; with the signs on the integer pipe
 // and float-stepped grid indices 448, the constants warp-uniform (RayC) and
 // four blocks per SM 406, the series two terms a step and pixels stepped
-// without divisions 388. The lens light in a loop of its own, so that its
+// without divisions 388, the series in straight-line code (Series) 367. The lens light in a loop of its own, so that its
 // eight accumulators are not live with the others: 412.
 //
 // F and the source position stay in Horner's form: next to the source's centre
@@ -743,35 +760,35 @@ __device__ __forceinline__ void light_adj(const RayLight& L, T px, T py, T g, T*
 // |u|^2 = |eps|^2 for every ray): two FMAs per term instead of four.
 // Branch-free: a ray inside rho < 1e-6 arcsec has S = 0, which zeroes its
 // deflection and every EPL derivative (all carry S).
-template <class T>
-__device__ __forceinline__ void ray_adj(const RayC& V, const float4* ser, T x, T y, T g, T* acc) {
-  T qx, qy;
-  light_adj(V.light[0], x, y, g, acc + A_L, qx, qy);
+template <int NP, class T>
+__device__ __forceinline__ void ray_adj(const RayC& V, const Series<NP, true>& ser, T x, T y, T g, T* acc) {
+  T gx, gy;
+  light_adj<false>(V.light[0], x, y, g, acc + A_L, gx, gy);
 
   const T dx = x - sp<T>(V.xc), dy = y - sp<T>(V.yc);
   const T wr = fmaT(sp<T>(-V.e1), dx, fmaT(sp<T>(-V.e2), dy, dx));
   const T wi = fmaT(sp<T>(V.e1), dy, fmaT(sp<T>(-V.e2), dx, dy));
   const T w2 = fmaT(wr, wr, wi * wi);
-  const T keep = geT(w2, sp<T>(V.w2min));
   const T w2c = maxT(w2, sp<T>(V.w2min));   // > 0; where it clamps, S = 0 zeroes every EPL term
   const T lrho = fmaT(sp<T>(-0.5f), lg2T(w2c), sp<T>(V.lc));  // log2(thetaE / rho)
-  const T S = keep * ex2T(fmaT(sp<T>(V.t), lrho, sp<T>(V.tlc_lo)));
+  const T S = where_ge(w2, sp<T>(V.w2min), ex2T(fmaT(sp<T>(V.t), lrho, sp<T>(V.tlc_lo))));
   const T iw2 = rcpT(w2c);
   const T nwi = -wi;
   const T vr = fmaT(wr, wr, nwi * wi) * iw2;
-  const T vi = sp<T>(2.f) * wr * wi * iw2;
-  const T ur = fmaT(sp<T>(-V.e1), vr, sp<T>(-V.e2) * vi);
-  const T ui = fmaT(sp<T>(V.e2), vr, sp<T>(-V.e1) * vi);
-  const T nui = fmaT(sp<T>(-V.e2), vr, sp<T>(V.e1) * vi);   // -ui: packed FMAs take no negated operands
+  const T vh = wr * wi * iw2;               // Im v / 2 (twice it goes into the constants: the same bits)
+  const T ur = fmaT(sp<T>(-V.e1), vr, sp<T>(-2.f * V.e2) * vh);
+  const T ui = fmaT(sp<T>(V.e2), vr, sp<T>(-2.f * V.e1) * vh);
+  const T nui = -ui;                        // packed FMAs take no negated operands
   const T ru = ur + ur, nu2 = sp<T>(-V.u2);
   // G = sum_{n<N} a_{n+1} u^n by Horner; dF/dt / ln 2 = sum_n b_n u^n = ur c1 - |u|^2 c2 + i ui c1;
   // the two highest terms start the sums, then two more per step
-  const float4 top = ser[V.npairs - 1];
+  const int np = NP > 0 ? NP : V.npairs;
+  const float4 top = ser.pair(np - 1);
   T Gr = fmaT(ur, sp<T>(top.y), sp<T>(top.x)), Gi = ui * sp<T>(top.y);
   T c2 = sp<T>(top.w), c1 = fmaT(ru, c2, sp<T>(top.z));
-#pragma unroll 1   // (unrolled by two: 388 -> 396 us; the coefficients as duplicated pairs in shared memory: 403)
-  for (int m = V.npairs - 2; m >= 0; --m) {
-    const float4 q = ser[m];
+#pragma unroll (NP > 0 ? SERIES_UNROLL : 1)
+  for (int m = np - 2; m >= 0; --m) {
+    const float4 q = ser.pair(m);
     const T n1 = fmaT(ur, Gr, fmaT(nui, Gi, sp<T>(q.y)));
     Gi = fmaT(ur, Gi, ui * Gr);
     c2 = fmaT(ru, c1, fmaT(nu2, c2, sp<T>(q.w)));
@@ -785,18 +802,14 @@ __device__ __forceinline__ void ray_adj(const RayC& V, const float4* ser, T x, T
   // (conj(1 - u) v = v + eps |v|^2, |v| = 1)
   const T nr = fmaT(sp<T>(V.th), hr, sp<T>(-V.kc) * Gr), ni = fmaT(sp<T>(V.th), hi, sp<T>(-V.kc) * Gi);
   const T idd = rcpT(sp<T>(V.den0) - ru);
-  const T er = (vr + sp<T>(V.e1)) * idd, ei = (vi + sp<T>(V.e2)) * idd;
+  const T er = (vr + sp<T>(V.e1)) * idd, ei = fmaT(sp<T>(2.f), vh, sp<T>(V.e2)) * idd;
   // lens equation with external shear, source at beta
-  const T swr = S * wr, swi = S * wi, nswi = S * nwi;   // S w
+  const T swr = S * wr, swi = S * wi, nswi = -swi;   // S w
   const T ar = fmaT(swr, hr, nswi * hi);
   const T ai = fmaT(swr, hi, swi * hr);
   const T bx = x - ar - fmaT(sp<T>(V.g1), x, sp<T>(V.g2) * y);
   const T by = y - ai - fmaT(sp<T>(V.g2), x, sp<T>(-V.g1) * y);
-  light_adj(V.light[1], bx, by, g, acc + A_S, qx, qy);
-  const RayLight& L = V.light[1];
-  const float Bh = 0.5f * L.B2;
-  const T gx = fmaT(sp<T>(L.A), qx, sp<T>(Bh) * qy);
-  const T gy = fmaT(sp<T>(Bh), qx, sp<T>(L.C) * qy);
+  light_adj<true>(V.light[1], bx, by, g, acc + A_S, gx, gy);
   const T ngy = -gy;
   acc[A_G1] = fmaT(gx, x, fmaT(ngy, y, acc[A_G1]));
   acc[A_G2] = fmaT(gx, y, fmaT(gy, x, acc[A_G2]));
@@ -817,12 +830,13 @@ __device__ __forceinline__ void ray_adj(const RayC& V, const float4* ser, T x, T
   acc[A_E2] = fmaT(Qr, dy, fmaT(nQi, dx, acc[A_E2] + Vi));
 }
 
-// Block size and resident blocks per SM of the adjoint kernel. Four blocks of
-// 128 threads (128 registers, 16 bytes of spills) against three (164, none) and
-// two: 406, 428 and 450 us at 60 x 60, k = 2, B = 4096; 535, 557 and 585 us at
-// 100 x 100, k = 4, B = 512; five (96 registers, 236 bytes of spills) 441 us.
+// Block size and resident blocks per SM of the adjoint kernel. With the series
+// in straight-line code, three blocks of 128 threads (168 registers, no
+// spills) against four (128, some 100 bytes of spills in each length's code):
+// 367 and 378 us at 60 x 60, k = 2, B = 4096; 473 and 489 us at 100 x 100, k = 4,
+// B = 512. 160 x 3 393, 96 x 5 394, 192 x 2 389, 64 x 7 384, 64 x 6 376 us.
 constexpr int ADJ_THREADS = 128;
-constexpr int ADJ_BLOCKS_PER_SM = 4;
+constexpr int ADJ_BLOCKS_PER_SM = 3;
 
 template <class Src>
 __global__ void __launch_bounds__(ADJ_THREADS, ADJ_BLOCKS_PER_SM) k_ray_adj(const __grid_constant__ Src src) {
@@ -850,42 +864,45 @@ __global__ void __launch_bounds__(ADJ_THREADS, ADJ_BLOCKS_PER_SM) k_ray_adj(cons
     const float* gpre = ss.work + size_t(b) * HW;
     if (sv.nterms >= 0) {
       const RayC rc = ray_consts(sv);
-      const int stride = blockDim.x;
-      // whole steps: two pixels per thread (p and p + blockDim), their rays paired in f32x2
-      const int nfull = (p1 - p0) / (2 * stride);
-      const PixelStep step(2 * stride, W);
-      int p = p0 + threadIdx.x;
-      int ip = p / W, jp = p - ip * W, iq = (p + stride) / W, jq = p + stride - iq * W;
-      for (int it = 0; it < nfull; ++it, p += 2 * stride, step.advance(ip, jp, W), step.advance(iq, jq, W)) {
-        const F2 g = {make_float2(gpre[p], gpre[p + stride])};
-        // grid indices of the pixels' first subpixels; a subpixel step adds 2
-        const F2 nx0 = {make_float2(float(2 * jp * k + ss.nx0), float(2 * jq * k + ss.nx0))};
-        F2 ny = {make_float2(float(2 * ip * k + ss.ny0), float(2 * iq * k + ss.ny0))};
-        for (int a = 0; a < k; ++a, ny = ny + sp<F2>(2.f)) {
-          const F2 y = grid_coord2(ny, ss.hh, ss.hl);
-          F2 nx = nx0;
-          for (int c = 0; c < k; ++c, nx = nx + sp<F2>(2.f))
-            ray_adj(rc, sv.ser, grid_coord2(nx, ss.hh, ss.hl), y, g, acc);
+      with_series(rc.npairs, [&](auto np) {
+        const Series<decltype(np)::value, true> ser(sv.ser);
+        const int stride = blockDim.x;
+        // whole steps: two pixels per thread (p and p + blockDim), their rays paired in f32x2
+        const int nfull = (p1 - p0) / (2 * stride);
+        const PixelStep step(2 * stride, W);
+        int p = p0 + threadIdx.x;
+        int ip = p / W, jp = p - ip * W, iq = (p + stride) / W, jq = p + stride - iq * W;
+        for (int it = 0; it < nfull; ++it, p += 2 * stride, step.advance(ip, jp, W), step.advance(iq, jq, W)) {
+          const F2 g = {make_float2(gpre[p], gpre[p + stride])};
+          // grid indices of the pixels' first subpixels; a subpixel step adds 2
+          const F2 nx0 = {make_float2(float(2 * jp * k + ss.nx0), float(2 * jq * k + ss.nx0))};
+          F2 ny = {make_float2(float(2 * ip * k + ss.ny0), float(2 * iq * k + ss.ny0))};
+          for (int a = 0; a < k; ++a, ny = ny + sp<F2>(2.f)) {
+            const F2 y = grid_coord2(ny, ss.hh, ss.hl);
+            F2 nx = nx0;
+            for (int c = 0; c < k; ++c, nx = nx + sp<F2>(2.f))
+              ray_adj(rc, ser, grid_coord2(nx, ss.hh, ss.hl), y, g, acc);
+          }
         }
-      }
-      // the ragged end (fewer than 2 blockDim pixels): its rays two per thread and step,
-      // so that every thread takes a share; an odd last ray is paired with itself at zero weight
-      const int base = p0 + 2 * stride * nfull, kk = k * k;
-      const int nr = (p1 - base) * kk;
-      for (int r = 2 * int(threadIdx.x); r < nr; r += 2 * stride) {
-        const bool has2 = r + 1 < nr;
-        const int r2 = has2 ? r + 1 : r;
-        const int pa = base + r / kk, sa = r - (pa - base) * kk;
-        const int pb = base + r2 / kk, sb = r2 - (pb - base) * kk;
-        const int ia = pa / W, ja = pa - ia * W, ib = pb / W, jb = pb - ib * W;
-        const int aa = sa / k, ca = sa - aa * k, ab = sb / k, cb = sb - ab * k;
-        const F2 y = {make_float2(grid_coord(2 * (ia * k + aa) + ss.ny0, ss.hh, ss.hl),
-                                  grid_coord(2 * (ib * k + ab) + ss.ny0, ss.hh, ss.hl))};
-        const F2 x = {make_float2(grid_coord(2 * (ja * k + ca) + ss.nx0, ss.hh, ss.hl),
-                                  grid_coord(2 * (jb * k + cb) + ss.nx0, ss.hh, ss.hl))};
-        const F2 g = {make_float2(gpre[pa], has2 ? gpre[pb] : 0.f)};
-        ray_adj(rc, sv.ser, x, y, g, acc);
-      }
+        // the ragged end (fewer than 2 blockDim pixels): its rays two per thread and step,
+        // so that every thread takes a share; an odd last ray is paired with itself at zero weight
+        const int base = p0 + 2 * stride * nfull, kk = k * k;
+        const int nr = (p1 - base) * kk;
+        for (int r = 2 * int(threadIdx.x); r < nr; r += 2 * stride) {
+          const bool has2 = r + 1 < nr;
+          const int r2 = has2 ? r + 1 : r;
+          const int pa = base + r / kk, sa = r - (pa - base) * kk;
+          const int pb = base + r2 / kk, sb = r2 - (pb - base) * kk;
+          const int ia = pa / W, ja = pa - ia * W, ib = pb / W, jb = pb - ib * W;
+          const int aa = sa / k, ca = sa - aa * k, ab = sb / k, cb = sb - ab * k;
+          const F2 y = {make_float2(grid_coord(2 * (ia * k + aa) + ss.ny0, ss.hh, ss.hl),
+                                    grid_coord(2 * (ib * k + ab) + ss.ny0, ss.hh, ss.hl))};
+          const F2 x = {make_float2(grid_coord(2 * (ja * k + ca) + ss.nx0, ss.hh, ss.hl),
+                                    grid_coord(2 * (jb * k + cb) + ss.nx0, ss.hh, ss.hl))};
+          const F2 g = {make_float2(gpre[pa], has2 ? gpre[pb] : 0.f)};
+          ray_adj(rc, ser, x, y, g, acc);
+        }
+      });
     }
     // pairwise FP32 sums within the warp (GB300's FP64 pipe is narrow), FP64 across warps
 #pragma unroll
@@ -2293,30 +2310,32 @@ static int fwd_blocks_per_sm() {
 
 // Tiling of a B-vector call's rays: the tile count that minimises a model of
 // the two ray kernels' time. Per kernel, with R resident blocks per SM, a
-// tile costs its pixels plus TILE_RAYS rays of prologue; the call is whole
-// waves of R blocks per SM and a part of one, which takes its share of a
-// wave but at least PART of one (fewer warps hide less latency), and a tail:
-// the last blocks of a mixed batch (drawn from a prior) end at different
-// times, TAIL_MIXED of a tile; below one vector per SM, near one mode, they
-// end together. The adjoint weighs 2, its time over the forward's. Measured,
-// forward + adjoint in us by tile count: 300 vectors of 80 x 80 from the prior
-// 1: 223, 2: 138, 3: 124, 4: 115, 6: 116, 8: 116 (takes 6); 50 vectors near one
-// mode 3: 43, 6: 34, 9: 31, 12: 31, 18: 35, 25: 34 (takes 9); 512 vectors of
-// 100 x 100, k = 4, 1: 980, 2: 836, 4: 814, 8: 799 (takes 8). A larger count must
-// gain two percent. Tiles keep at least one step of a block (two pixels a
-// thread) and four rays a thread.
+// tile costs its pixels plus TILE_RAYS rays of prologue, and the call is whole
+// waves of R blocks per SM and a part f of one. A part after whole waves
+// costs more than its share (min(1, 0.08 + 1.22 f): 1024 vectors of 200 x 200,
+// k = 4, k_ray_adj 3984, 3868, 3846, 3737, 3760 us at 1, 2, 3, 4, 8 tiles, that
+// is 2.25, 4.49, 6.74, 8.98, 17.97 waves), and a lone part too (0.2 + 0.8 f:
+// fewer warps hide less latency). From one vector per SM on, a batch may mix
+// short and long series, and its longest block ends late: TAIL of a tile
+// (2000 prior draws of 80 x 80, log L alone, k_ray_fwd at 1, 2, 3 tiles 1.15,
+// 1.00, 1.01 of the best). The adjoint weighs 2, its time over the forward's. Forward +
+// adjoint by tile count: 300 prior draws of 80 x 80 2: 119, 3: 106, 4: 103.5, 6:
+// 104, 8: 106, 12: 114 us; 50 vectors near one mode 6: 29.8, 9: 30.3, 12: 30.0, 15:
+// 32.3; 512 vectors of 100 x 100, k = 4, 1: 797, 2: 683, 4: 682, 8: 679, 12: 699. A
+// larger count must gain 1.5%. Tiles keep at least one step of a block (two
+// pixels a thread) and four rays a thread.
 struct TilePlan {
   int ntiles, tile_pix;
 };
 
 static double ray_kernel_cost(double items, double px, double slots, double tail) {
-  constexpr double PART = 0.55;
-  const double w = items / slots, full = std::floor(w), part = w - full;
-  return px * (full + (part > 0.0 ? (part > PART ? part : PART) : 0.0) + tail);
+  const double w = items / slots, full = std::floor(w), f = w - full;
+  const double part = f <= 0.0 ? 0.0 : full > 0.0 ? std::fmin(1.0, 0.08 + 1.22 * f) : 0.2 + 0.8 * f;
+  return px * (full + part + tail);
 }
 
 static TilePlan plan_rays(int B, int H, int W, int k) {
-  constexpr double TILE_RAYS = 256.0, TAIL_MIXED = 0.35, TAIL_MODE = 0.1;
+  constexpr double TILE_RAYS = 400.0, TAIL = 0.25;
   const int HW = H * W;
   TilePlan best{1, HW};
   if (B <= 0 || HW <= 0) return best;
@@ -2325,10 +2344,10 @@ static TilePlan plan_rays(int B, int H, int W, int k) {
   const long long by_rays = (rays + 4 * ADJ_THREADS - 1) / (4 * ADJ_THREADS);
   if (by_rays < max_nt) max_nt = by_rays;
   const double sms = num_sms(), fwd_slots = sms * fwd_blocks_per_sm(), adj_slots = sms * ADJ_BLOCKS_PER_SM;
-  const long long by_waves = (long long)(8.0 * adj_slots / B);   // past eight waves a finer tiling evens out nothing
+  const long long by_waves = (long long)(16.0 * adj_slots / B);   // past sixteen waves a finer tiling evens out nothing
   if (by_waves < max_nt) max_nt = by_waves;
   if (max_nt < 1) max_nt = 1;
-  const double tail = B < sms ? TAIL_MODE : TAIL_MIXED;
+  const double tail = B < sms ? 0.0 : TAIL;
   double best_cost = 0.0;
   for (long long nt = 1; nt <= max_nt; ++nt) {
     const int tp = int((HW + nt - 1) / nt);
@@ -2337,7 +2356,7 @@ static TilePlan plan_rays(int B, int H, int W, int k) {
     const double items = double(B) * ntt, px = tp + TILE_RAYS / (double(k) * k);
     const double cost = ray_kernel_cost(items, px, fwd_slots, tail) * fwd_slots / adj_slots +
                         2.0 * ray_kernel_cost(items, px, adj_slots, tail);
-    if (nt == 1 || cost < best_cost * 0.98) {
+    if (nt == 1 || cost < best_cost * 0.985) {
       best_cost = cost;
       best = TilePlan{ntt, tp};
     }
