@@ -2021,16 +2021,18 @@ __global__ void __launch_bounds__(BAND_THREADS, 2) k_conv_sep_bands(const __grid
 
 // The per-vector chain rule: gradient entry j from the summed accumulators
 // a[NACC] (Acc: what each holds) is, in FP64,
-//   scale_j (k0 a[i0] + k1 a[i1] + k2 a[i2])
-// (n1 .. of the terms used). The terms are set up per entry from the
-// parameters pf and the constants V, without FP64 divisions except for the
-// one reciprocal, so that lanes of a warp that form different entries only
-// diverge over cheap FP32 and index selects, and the loads and the
-// reciprocal do not wait for the accumulators. Shared by the two k_final
-// variants so that they give identical results.
+//   scale_j (k0 a[i0] + k1 a[i1] + k2 a[i2]),
+// unused terms with k = 0 and an accumulator that the entry uses anyway. The
+// coefficients are selected in FP32 (all but a few are floats) and every
+// entry runs the same FP64 operations: that pipe takes a warp instruction in
+// sixteen clocks, and lanes that diverge over the entries' own formulas
+// serialise on it (50 vectors, k_final_warp 10.5 us with a branch per kind of
+// entry, 8.3 us so). The terms and the reciprocal do not wait for the
+// accumulators. Shared by the two k_final variants so that they give identical
+// results.
 struct ChainTerm {
   double scale, k[3];
-  int i[3], n;
+  int i[3];
 };
 // The parameter n of the light whose b_n / n = 1.9992 - 0.3271 / n entry j
 // takes: the source's for the mass parameters.
@@ -2039,64 +2041,36 @@ __device__ __forceinline__ int chain_recip_param(int j) { return j >= 8 && j < 1
 // rn: 1 / pf[chain_recip_param(j)]; r2: 1 / thetaE, 1 / R_l, 1 / R_s for entries 0, 8 and 15
 __device__ __forceinline__ ChainTerm chain_term(int j, const float* pf, const VecConst& V, double rn, double r2) {
   const double ln2 = 0.69314718055994530942;
-  const bool lens = j >= 8 && j < 15;
-  const double I0 = pf[lens ? 14 : 21];
+  const bool mass = j < 8, lens = j >= 8 && j < 15;
+  const int l = lens ? 0 : 1, o = lens ? int(A_L) : int(A_S), k = mass ? -1 : j - (lens ? 8 : 15);
+  const LightC& L = V.light[l];
+  const float e1 = pf[2], e2 = pf[3];
+  const double I0 = pf[lens ? 14 : 21], t = double(pf[1]) - 1.0;
   const double bn = fma(-0.3271, rn, 1.9992);   // b_n / n
   const double m = bn * I0;
   ChainTerm c;
-  c.k[0] = 1.0;
-  c.k[1] = c.k[2] = 0.0;
-  c.i[1] = c.i[2] = 0;
-  c.n = 1;
-  if (j < 8) {
-    const double t = double(pf[1]) - 1.0, e1 = pf[2], e2 = pf[3];
-    c.scale = j == 0 ? m * t * r2 : j == 1 ? m * ln2 : j < 4 ? -m : m;
-    c.i[0] = j < 4 ? j : j < 6 ? int(A_QR) : j;
-    if (j == 2 || j == 3) {
-      c.n = 2;
-      c.i[1] = A_THETAE;
-      c.k[1] = t * double(j == 2 ? V.e1i : V.e2i);
-    } else if (j == 4 || j == 5) {
-      c.n = 2;
-      c.k[0] = j == 4 ? e1 - 1.0 : e2;
-      c.i[1] = A_QI;
-      c.k[1] = j == 4 ? -e2 : e1 + 1.0;
-    }
-    return c;
-  }
-  const int o = lens ? int(A_L) : int(A_S), k = j - (lens ? 8 : 15);
-  const LightC& L = V.light[lens ? 0 : 1];
-  c.scale = k == 0 ? m * r2 : k == 1 ? I0 : k < 4 ? -0.5 * m : k < 6 ? m : 1.0;
-  c.i[0] = o + (k == 0 ? 0 : k == 1 ? 1 : k < 4 ? 4 : k < 6 ? 2 : 7);
-  if (k == 1) {
-    c.n = 3;
-    c.k[0] = ln2 * bn;
-    c.i[1] = o + 7;
-    c.k[1] = 1.9992;
-    c.i[2] = o;
-    c.k[2] = -1.9992;
-  } else if (k == 2 || k == 3) {
-    c.n = 3;
-    c.k[0] = k == 2 ? L.A1 : L.A2;
-    c.i[1] = o + 5;
-    c.k[1] = k == 2 ? L.B21 : L.B22;
-    c.i[2] = o + 6;
-    c.k[2] = k == 2 ? L.C1 : L.C2;
-  } else if (k == 4 || k == 5) {
-    const float Bh = 0.5f * L.B2;
-    c.n = 2;
-    c.k[0] = k == 4 ? L.A : Bh;
-    c.i[1] = o + 3;
-    c.k[1] = k == 4 ? Bh : L.C;
-  }
+  // the accumulators of the three terms
+  c.i[0] = mass ? (j == 4 || j == 5 ? int(A_QR) : j) : o + (k == 0 ? 0 : k == 1 ? 1 : k < 4 ? 4 : k < 6 ? 2 : 7);
+  c.i[1] = j == 2 || j == 3 ? int(A_THETAE) : j == 4 || j == 5 ? int(A_QI)
+           : k == 1 ? o + 7 : k == 2 || k == 3 ? o + 5 : k == 4 || k == 5 ? o + 3 : c.i[0];
+  c.i[2] = j == 4 ? int(A_QR) : j == 5 ? int(A_QI) : k == 1 ? o : k == 2 || k == 3 ? o + 6 : c.i[0];
+  // their coefficients as floats
+  const float Bh = 0.5f * L.B2;
+  const float f0 = j == 4 ? e1 : j == 5 ? e2 : k == 2 ? L.A1 : k == 3 ? L.A2 : k == 4 ? L.A : k == 5 ? Bh : 1.f;
+  const float f1 = j == 2 ? V.e1i : j == 3 ? V.e2i : j == 4 ? -e2 : j == 5 ? e1
+                   : k == 2 ? L.B21 : k == 3 ? L.B22 : k == 4 ? Bh : k == 5 ? L.C : 0.f;
+  const float f2 = j == 4 ? -1.f : j == 5 ? 1.f : k == 2 ? L.C1 : k == 3 ? L.C2 : 0.f;
+  c.k[0] = k == 1 ? ln2 * bn : double(f0);
+  c.k[1] = k == 1 ? 1.9992 : double(f1) * (mass ? (j < 4 ? t : 1.0) : 1.0);
+  c.k[2] = k == 1 ? -1.9992 : double(f2);
+  const double base = k == 1 ? I0 : k == 6 ? 1.0 : m;
+  const double unit = j == 1 ? ln2 : j == 2 || j == 3 ? -1.0 : k == 2 || k == 3 ? -0.5 : 1.0;
+  c.scale = base * (j == 0 ? t * r2 : k == 0 ? r2 : unit);
   return c;
 }
 
 __device__ __forceinline__ double chain_rule(const ChainTerm& c, const double* a) {
-  double v = c.k[0] * a[c.i[0]];
-  if (c.n > 1) v = fma(c.k[1], a[c.i[1]], v);
-  if (c.n > 2) v = fma(c.k[2], a[c.i[2]], v);
-  return c.scale * v;
+  return c.scale * fma(c.k[2], a[c.i[2]], fma(c.k[1], a[c.i[1]], c.k[0] * a[c.i[0]]));
 }
 
 // One thread per vector (calls whose vectors have one ray tile each).
@@ -2445,10 +2419,10 @@ static cudaError_t launch_conv_class(int cls, const Src& src, int nitems, size_t
                   : launch_conv<11, 256, 3>(src, nitems, smem, mode, st, persistent);
     case 1:
       return wide ? launch_conv<21, 512, 1>(src, nitems, smem, mode, st, persistent)
-                  : launch_conv<21, 256, 1>(src, nitems, smem, mode, st, persistent);
+                  : launch_conv<21, 256, 2>(src, nitems, smem, mode, st, persistent);
     default:
       return wide ? launch_conv<0, 512, 1>(src, nitems, smem, mode, st, persistent)
-                  : launch_conv<0, 256, 2>(src, nitems, smem, mode, st, persistent);
+                  : launch_conv<0, 256, 3>(src, nitems, smem, mode, st, persistent);
   }
 }
 
@@ -2746,10 +2720,10 @@ cudaError_t prepare_devtable(const size_t* conv_smem) {
                                         : set_devtable_attr<11, 256, 3>(conv_smem[0]);
   if (e != cudaSuccess) return e;
   e = conv_smem[1] > CONV_WIDE_MIN_SMEM ? set_devtable_attr<21, 512, 1>(conv_smem[1])
-                                        : set_devtable_attr<21, 256, 1>(conv_smem[1]);
+                                        : set_devtable_attr<21, 256, 2>(conv_smem[1]);
   if (e != cudaSuccess) return e;
   return conv_smem[2] > CONV_WIDE_MIN_SMEM ? set_devtable_attr<0, 512, 1>(conv_smem[2])
-                                           : set_devtable_attr<0, 256, 2>(conv_smem[2]);
+                                           : set_devtable_attr<0, 256, 3>(conv_smem[2]);
 }
 
 cudaError_t launch_devtable(const TableHdr* d_hdr, const Seg* d_segs, const size_t* conv_smem, cudaStream_t st,
