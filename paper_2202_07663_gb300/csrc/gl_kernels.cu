@@ -1418,9 +1418,16 @@ __device__ __forceinline__ SepLayout sep_layout(const Seg& s, float* smem, int r
   return L;
 }
 
-// The factors into shared memory and the input buffer's halo (everything
-// outside rows c .. c + H - 1, columns c .. c + W - 1) zeroed; rows across
-// warps, columns across lanes. The caller synchronises the block before
+// Whether the horizontal passes of a whole image leave out the rows outside
+// it (of zeros): where that saves a group of 32 rows. Zeroing those rows of the
+// row buffers beforehand costs a little: 60 x 60, K = 11 (2 groups for 3), B =
+// 4096, k_conv_sep 91 -> 87 us, but 80 x 80 (3 for 3), B = 500, 28.6 -> 30.7.
+__device__ __forceinline__ bool sep_image_rows_only(int H, int Ht) { return ((H + 31) >> 5) < ((Ht + 31) >> 5); }
+
+// The factors into shared memory, and zeros into the input buffer's halo
+// (everything outside rows c .. c + H - 1, columns c .. c + W - 1) and into the
+// row buffers' rows outside the image where the horizontal passes leave them
+// alone; rows across warps, columns across lanes. The caller synchronises the block before
 // the factors are read.
 __device__ __forceinline__ void sep_prepare(const Seg& s, const SepLayout& L) {
   const int K = s.K, c = (K - 1) / 2;
@@ -1433,8 +1440,11 @@ __device__ __forceinline__ void sep_prepare(const Seg& s, const SepLayout& L) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
   for (int i = wid; i < L.Ht; i += nw) {
     const bool inner = i >= c && i < c + s.H;
-    for (int q = lane; q < L.P; q += 32)
+    for (int q = lane; q < L.P; q += 32) {
       if (!inner || q < c || q >= c + s.W) L.img[i * L.P + q] = 0.f;
+      if (!inner && sep_image_rows_only(s.H, L.Ht))
+        for (int r = 0; r < R; ++r) L.tmp[(size_t(r) * L.Ht + i) * L.P + q] = 0.f;
+    }
   }
 }
 
@@ -1472,26 +1482,28 @@ __device__ __forceinline__ void sep_htaps(const float* __restrict__ in, const fl
   }
 }
 
-// Horizontal passes: row buffer r, row i, columns j0 .. j0 + 15, for the Ht
-// rows. A warp takes 32 consecutive rows of one strip (float4 loads of rows
-// an odd number of 16-byte words apart are conflict-free). FLIP: the flipped
+// Horizontal passes: row buffer r, row i, columns j0 .. j0 + 15, for the rows
+// row0 .. row0 + nrows - 1. A warp takes 32 consecutive rows of one strip
+// (float4 loads of rows an odd number of 16-byte words apart are
+// conflict-free). FLIP: the flipped
 // factor (the model's convolution); RC: the rank when known at compile time
 // (1), else 0. K == 0: any odd side Kk, in groups of 8 taps.
 template <int K, bool FLIP, int RC>
-__device__ __forceinline__ void sep_hpass(const float* __restrict__ in, const SepLayout& L, int W, int Rrt, int Kk) {
+__device__ __forceinline__ void sep_hpass(const float* __restrict__ in, const SepLayout& L, int W, int Rrt, int Kk,
+                                          int row0, int nrows) {
   constexpr int S = 16;
   const int R = RC > 0 ? RC : Rrt;
-  const int P = L.P, Ht = L.Ht, nstrip = (W + S - 1) / S, rg = (Ht + 31) >> 5, tasks = nstrip * rg;
+  const int P = L.P, Ht = L.Ht, nstrip = (W + S - 1) / S, rg = (nrows + 31) >> 5, tasks = nstrip * rg;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
   int strip = wid / rg, g = wid - strip * rg;   // task w = strip * rg + g, stepped without division
   for (int w = wid; w < tasks; w += nw) {
-    const int i = g * 32 + lane, j0 = strip * S;
+    const int i = row0 + g * 32 + lane, j0 = strip * S;
     g += nw;
     while (g >= rg) {
       g -= rg;
       ++strip;
     }
-    if (i >= Ht) continue;
+    if (i >= row0 + nrows) continue;
     const float* row = in + i * P + j0;
     for (int r = 0; r < R; ++r) {
       float acc[S];
@@ -1609,12 +1621,14 @@ __device__ void conv_vector_sep(const Seg& s, int b, int mode_rt, float* smem, d
   const bool corr_only = (mode == MODE_CORR);   // the work slot holds d log L / d M already
   const bool want_grad = (mode == MODE_GRAD) || corr_only;
   const int Wp2 = (W + 1) >> 1;
+  const bool image_rows = sep_image_rows_only(H, L.Ht);
+  const int row0 = image_rows ? c : 0, nrows = image_rows ? H : L.Ht;
   if (!prepared) sep_prepare(s, L);
   if (!PF) sep_load_issue(s, L, work);
   cp_async_wait_all();
   __syncthreads();
   if (!corr_only) {
-    sep_hpass<K, true, RC>(L.img, L, W, R, s.K);
+    sep_hpass<K, true, RC>(L.img, L, W, R, s.K, row0, nrows);
     __syncthreads();
     float ll = 0.f, c2 = 0.f;
     for_vunits(L.nvs, Wp2, [&](int i0, int j) {
@@ -1643,7 +1657,7 @@ __device__ void conv_vector_sep(const Seg& s, int b, int mode_rt, float* smem, d
     block_loglik(s, b, ll, c2, red2);   // also the barrier before the correlation reads img
     if (!want_grad) return;
   }
-  sep_hpass<K, false, RC>(L.img, L, W, R, s.K);
+  sep_hpass<K, false, RC>(L.img, L, W, R, s.K, row0, nrows);
   __syncthreads();
   if (PF && next_b >= 0) sep_load_issue(s, L, s.work + size_t(next_b) * HW);
   const float inv_k2 = 1.0f / float(s.k * s.k);
@@ -1932,7 +1946,7 @@ __global__ void __launch_bounds__(BAND_THREADS, 2) k_conv_sep_bands(const __grid
   __syncthreads();
   const int Wp2 = (W + 1) >> 1, nvu = ((nr + SEP_RV - 1) / SEP_RV) * Wp2;
   if (!corr_only) {
-    sep_hpass<K, true, 0>(L.img, L, W, R, s.K);
+    sep_hpass<K, true, 0>(L.img, L, W, R, s.K, 0, L.Ht);
     __syncthreads();
     float ll = 0.f, c2 = 0.f;
     for (int u = threadIdx.x; u < nvu; u += blockDim.x) {
@@ -2000,7 +2014,7 @@ __global__ void __launch_bounds__(BAND_THREADS, 2) k_conv_sep_bands(const __grid
   } else {
     cluster.sync();   // every band holds its input before any band writes the work slot
   }
-  sep_hpass<K, false, 0>(L.img, L, W, R, s.K);
+  sep_hpass<K, false, 0>(L.img, L, W, R, s.K, 0, L.Ht);
   __syncthreads();
   const float inv_k2 = 1.0f / float(s.k * s.k);
   for (int u = threadIdx.x; u < nvu; u += blockDim.x) {
@@ -2021,9 +2035,8 @@ __global__ void __launch_bounds__(BAND_THREADS, 2) k_conv_sep_bands(const __grid
 
 // The per-vector chain rule: gradient entry j from the summed accumulators
 // a[NACC] (Acc: what each holds) is, in FP64,
-//   scale_j (k0 a[i0] + k1 a[i1] + k2 a[i2]),
-// unused terms with k = 0 and an accumulator that the entry uses anyway. The
-// coefficients are selected in FP32 (all but a few are floats) and every
+//   scale_j (k0 a[i0] + k1 a[i1] + k2 a[i2])
+// (n: the terms used). The coefficients are selected in FP32 (all but a few are floats) and every
 // entry runs the same FP64 operations: that pipe takes a warp instruction in
 // sixteen clocks, and lanes that diverge over the entries' own formulas
 // serialise on it (50 vectors, k_final_warp 10.5 us with a branch per kind of
@@ -2032,7 +2045,7 @@ __global__ void __launch_bounds__(BAND_THREADS, 2) k_conv_sep_bands(const __grid
 // results.
 struct ChainTerm {
   double scale, k[3];
-  int i[3];
+  int i[3], n;
 };
 // The parameter n of the light whose b_n / n = 1.9992 - 0.3271 / n entry j
 // takes: the source's for the mass parameters.
@@ -2049,6 +2062,7 @@ __device__ __forceinline__ ChainTerm chain_term(int j, const float* pf, const Ve
   const double bn = fma(-0.3271, rn, 1.9992);   // b_n / n
   const double m = bn * I0;
   ChainTerm c;
+  c.n = j == 2 || j == 3 ? 2 : j == 4 || j == 5 ? 3 : k >= 1 && k < 4 ? 3 : k == 4 || k == 5 ? 2 : 1;
   // the accumulators of the three terms
   c.i[0] = mass ? (j == 4 || j == 5 ? int(A_QR) : j) : o + (k == 0 ? 0 : k == 1 ? 1 : k < 4 ? 4 : k < 6 ? 2 : 7);
   c.i[1] = j == 2 || j == 3 ? int(A_THETAE) : j == 4 || j == 5 ? int(A_QI)
@@ -2070,7 +2084,10 @@ __device__ __forceinline__ ChainTerm chain_term(int j, const float* pf, const Ve
 }
 
 __device__ __forceinline__ double chain_rule(const ChainTerm& c, const double* a) {
-  return c.scale * fma(c.k[2], a[c.i[2]], fma(c.k[1], a[c.i[1]], c.k[0] * a[c.i[0]]));
+  double v = c.k[0] * a[c.i[0]];
+  if (c.n > 1) v = fma(c.k[1], a[c.i[1]], v);
+  if (c.n > 2) v = fma(c.k[2], a[c.i[2]], v);
+  return c.scale * v;
 }
 
 // One thread per vector (calls whose vectors have one ray tile each).
