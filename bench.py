@@ -43,19 +43,20 @@ WORKLOAD = inputs.MULTISTART
 # FP32 flop counts per ray of the two ray kernels (FMA = 2), N = EPL series
 # terms of the vector; per pixel of the convolution kernel.
 def flops_ray_fwd(N):
-    return 90 + 7 * N
+    return 85 + 7 * N
 
 
 def flops_ray_adj(N):
-    return 331 + 14 * N
+    return 184 + 11 * N
 
 
 def flops_conv_pixel(K, grad, R=0):
-    """K x K stencil: 2 K^2 flops per pass; R separable terms: a K-tap
-    horizontal and a K-tap vertical pass per term, 4 K R flops per pass.
-    Two passes (model, adjoint correlation) with the gradient; ~25 for the
+    """K x K stencil: the workloads' PSFs mirror, so the two input rows of a
+    kernel row are added first, K (K + 1) + K flops per pass; R separable
+    terms: a K-tap horizontal and a K-tap vertical pass per term, 4 K R flops
+    per pass. Two passes (model, adjoint correlation) with the gradient; ~25 for the
     likelihood terms."""
-    per_pass = 4 * K * R if R > 0 else 2 * K * K
+    per_pass = 4 * K * R if R > 0 else K * (K + 1) + K
     return (2 if grad else 1) * per_pass + 25
 
 
@@ -87,7 +88,7 @@ def series_terms(params: np.ndarray, adjoint: bool) -> np.ndarray:
     return first.astype(np.int64)
 
 
-MUFU_RAY_ADJ = 13   # ex2/lg2/rcp per ray in the adjoint: EPL 5 (lg2, ex2, three rcp), each Sersic profile 4
+MUFU_RAY_ADJ = 12   # ex2/lg2/rcp per ray in the adjoint: EPL 4 (lg2, ex2, two rcp), each Sersic profile 4
 # DRAM bytes per launch of k_ray_adj from one ncu capture, keyed by workload
 # and the kernel source it was taken on (sha256 prefix of gl_kernels.cu +
 # gl_device.cuh); any other source reports null traffic until it is captured again.

@@ -115,7 +115,7 @@ int gl_system_create_obsvar(gl_system** out, const float* image, const float* no
  *   device). The convolution of Eq. 4's model (and its adjoint) with a PSF
  *   P = sum_{r<R} u_r v_r^T is R pairs of 1-D passes, 2 K R multiply-adds per
  *   pixel instead of K^2. gl_system_create applies this to its PSF: when
- *   R > 0 and the PSF side is 11 or 21 it keeps the factors
+ *   0 < R <= K / 4 it keeps the factors
  *   (gl_system_psf_rank) and convolves that way, the whole image in one
  *   block when its R + 1 padded buffers fit 200 KiB of shared memory
  *   ((R + 1) * (ceil(H/8)*8 + K - 1) * P * 4 bytes, P as below), else (and

@@ -9,8 +9,8 @@
 //              Gaussian log-likelihood term, FP64 block reduction -> log L;
 //              for the gradient also the pixel adjoint d log L / d I_model,
 //              correlated with the PSF and divided by k^2 -> work
-//   k_ray_adj  per (vector, pixel tile): rays recomputed, forward-mode
-//              derivatives contracted with the subpixel adjoint -> partial
+//   k_ray_adj  per (vector, pixel tile): rays recomputed, the subpixel adjoint
+//              carried back through each to 24 sums -> partial
 //   k_final    per vector: fixed-order FP64 sum of the tile partials and the
 //              per-vector chain rule -> grad
 // Every kernel loops over its items with a grid stride, so the same code
