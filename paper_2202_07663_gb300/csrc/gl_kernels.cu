@@ -2646,7 +2646,8 @@ static cudaError_t launch_conv_single(const OneSeg& src, int mode, cudaStream_t 
   int rows = 0;
   const bool small = 2 * s.B <= num_sms();
   const int sb = s.psf_rank > 0 && (small || !s.conv_sep) ? sep_band_plan(s.H, s.W, s.K, s.psf_rank, small, s.B, &rows) : 0;
-  const int nb = (sb > 0 || s.conv_sep) ? 0 : conv_bands(s.B, s.H, s.W, s.K);
+  // (an image that only fits as column strips keeps their summation order, as in grouped calls)
+  const int nb = (sb > 0 || s.conv_sep || !s.conv_rows) ? 0 : conv_bands(s.B, s.H, s.W, s.K);
   cudaError_t e;
   if (sb > 0)
     e = s.K == 11   ? launch_conv_sep_bands<11>(src, sb, rows, mode, st)
