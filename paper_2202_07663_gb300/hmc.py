@@ -76,14 +76,17 @@ def _fused_vjp(in_dtype, grad_out, g) -> bool:
     """Whether the gradient rows are scaled by the library's kernel: plain
     float32 CUDA gradients, and nothing that has to see the product as torch
     operations (a gradient of the gradient; a batched, transformed or
-    subclassed tensor, which has no storage of its own or another type; a saved
-    gradient that a hook has moved or changed)."""
+    subclassed tensor, which has no storage of its own or another type; one
+    whose memory is not its values, as the imaginary part of a conjugate holds
+    them negated and a zero tensor none; a saved gradient that a hook has moved
+    or changed)."""
     return (in_dtype == torch.float32 and not torch.is_grad_enabled()
             and type(grad_out) is torch.Tensor and type(g) is torch.Tensor
             and grad_out.dtype == torch.float32 and g.dtype == torch.float64 and grad_out.is_cuda
             and grad_out.device == g.device and g.device.index == torch.cuda.current_device()
             and grad_out.shape == g.shape[:1] and grad_out.stride(0) >= 0 and g.is_contiguous() and g.numel() > 0
-            and torch._C._has_storage(grad_out))
+            and torch._C._has_storage(grad_out) and not grad_out._is_zerotensor()
+            and not grad_out.is_neg() and not g.is_neg())
 
 
 def loglik(params, system):

@@ -68,3 +68,28 @@ def test_other_uses_keep_the_torch_expression(setup):
         ll = hmc.loglik(p, s)
     (out,) = torch.autograd.grad(ll.sum(), p)
     assert torch.equal(out, g.to(torch.float32))
+
+
+def _expression(go, g):
+    return (go.to(torch.float64)[:, None] * g).to(torch.float32)
+
+
+def test_incoming_gradient_whose_memory_holds_its_negative(setup):
+    """The imaginary part of a conjugate is a view of the unconjugated memory
+    with torch's negative bit; given as grad_outputs and as the engine forms it
+    for a complex function of log L. A zero tensor has no memory at all."""
+    hmc, s, p0 = setup
+    p = p0.clone().requires_grad_()
+    g = s.loglik_grad(p0)[1]
+    z = torch.complex(torch.randn(len(p0), device="cuda"), torch.randn(len(p0), device="cuda"))
+    go = z.conj().imag
+    assert go.is_neg()
+    (out,) = torch.autograd.grad(hmc.loglik(p, s), p, grad_outputs=go)
+    assert torch.equal(out, _expression(-z.imag, g))
+    ll = hmc.loglik(p, s)
+    value = (torch.complex(torch.zeros_like(ll), ll).conj() * z.conj()).imag.sum()
+    (go,) = torch.autograd.grad(value, ll, retain_graph=True)
+    (out,) = torch.autograd.grad(value, p)
+    assert torch.equal(out, _expression(-z.real, g)) and torch.equal(out, _expression(go, g))
+    (out,) = torch.autograd.grad(hmc.loglik(p, s), p, grad_outputs=torch._efficientzerotensor((len(p0),), device="cuda"))
+    assert torch.equal(out, torch.zeros_like(out))
