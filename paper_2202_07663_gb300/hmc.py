@@ -62,6 +62,9 @@ class LogLik(torch.autograd.Function):
     @staticmethod
     def backward(ctx, grad_out):
         (g,) = ctx.saved_tensors
+        if grad_out.layout is not torch.strided:
+            # (gather with sparse_grad=True) a sparse column times the rows would fill the first entry only
+            grad_out = grad_out.to_dense()
         if _fused_vjp(ctx.in_dtype, grad_out, g):
             # one launch in place of two casts and a product (the same numbers): a backward
             # pass over a batch this small is host time, 64 -> 36 us of it for 160 vectors

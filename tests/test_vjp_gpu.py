@@ -93,3 +93,16 @@ def test_incoming_gradient_whose_memory_holds_its_negative(setup):
     assert torch.equal(out, _expression(-z.real, g)) and torch.equal(out, _expression(go, g))
     (out,) = torch.autograd.grad(hmc.loglik(p, s), p, grad_outputs=torch._efficientzerotensor((len(p0),), device="cuda"))
     assert torch.equal(out, torch.zeros_like(out))
+
+
+def test_sparse_incoming_gradient(setup):
+    """gather(sparse_grad=True) on log L sends back a sparse gradient: the rows
+    of the gathered vectors, whole."""
+    hmc, s, p0 = setup
+    p = p0.clone().requires_grad_()
+    g = s.loglik_grad(p0)[1]
+    rows = torch.tensor([1, 5, 20], device="cuda")
+    (out,) = torch.autograd.grad(torch.gather(hmc.loglik(p, s), 0, rows, sparse_grad=True).sum(), p)
+    ref = torch.zeros(g.shape, device="cuda")
+    ref[rows] = g[rows].to(torch.float32)
+    assert torch.equal(out, ref)
