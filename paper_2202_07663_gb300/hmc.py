@@ -78,12 +78,12 @@ class LogLik(torch.autograd.Function):
 def _fused_vjp(in_dtype, grad_out, g) -> bool:
     """Whether the gradient rows are scaled by the library's kernel: plain
     float32 CUDA gradients, and nothing that has to see the product as torch
-    operations (a gradient of the gradient; a batched, transformed or
+    operations (a gradient of the gradient; a dispatch mode; a batched, transformed or
     subclassed tensor, which has no storage of its own or another type; one
     whose memory is not its values, as the imaginary part of a conjugate holds
     them negated and a zero tensor none; a saved gradient that a hook has moved
     or changed)."""
-    return (in_dtype == torch.float32 and not torch.is_grad_enabled()
+    return (in_dtype == torch.float32 and not torch.is_grad_enabled() and not torch._C._len_torch_dispatch_stack()
             and type(grad_out) is torch.Tensor and type(g) is torch.Tensor
             and grad_out.dtype == torch.float32 and g.dtype == torch.float64 and grad_out.is_cuda
             and grad_out.device == g.device and g.device.index == torch.cuda.current_device()

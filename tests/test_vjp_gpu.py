@@ -106,3 +106,24 @@ def test_sparse_incoming_gradient(setup):
     ref = torch.zeros(g.shape, device="cuda")
     ref[rows] = g[rows].to(torch.float32)
     assert torch.equal(out, ref)
+
+
+def test_dispatch_mode_sees_the_product(setup):
+    """A dispatch mode (a tracer, an operation counter) that is active during
+    the backward pass gets the product as torch operations."""
+    from torch.utils._python_dispatch import TorchDispatchMode
+    hmc, s, p0 = setup
+    seen = []
+
+    class Record(TorchDispatchMode):
+        def __torch_dispatch__(self, func, types, args=(), kwargs=None):
+            seen.append(str(func))
+            return func(*args, **(kwargs or {}))
+
+    p = p0.clone().requires_grad_()
+    ll = hmc.loglik(p, s)
+    w = torch.randn(len(p0), device="cuda")
+    with Record():
+        (out,) = torch.autograd.grad(ll, p, grad_outputs=w)
+    assert any(name.startswith("aten.mul") for name in seen)
+    assert torch.equal(out, _expression(w, s.loglik_grad(p0)[1]))
