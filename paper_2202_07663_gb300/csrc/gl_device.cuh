@@ -93,8 +93,7 @@ struct __align__(16) VecConst {
   float omt;               // 1 - t
   float e1i, e2i;          // e1, e2 times 1 / (1 - |eps|^2)
   int order;               // written by k_order into slot p: the vector the ray kernels take p-th
-  float den0;              // 1 + |eps|^2: |1 - u|^2 = den0 - 2 Re u
-  float pad_[2];
+  float pad_[3];
   LightC light[2];         // [0] lens light at theta, [1] source at beta
   // the series two terms at a time: (a_{2m+1}, a_{2m+2}, b_{2m+1}, b_{2m+2}), a_n = c_1 ... c_n and
   // b_n = d a_n / d t / ln 2, zero past the term count
@@ -270,7 +269,7 @@ struct RayLight {
   float A, B2, C, x, y, c1, r2min, k1, I0;
 };
 struct RayC {
-  float xc, yc, e1, e2, lc, tlc_lo, t, w2min, g1, g2, th, kc, u2, omt, den0;
+  float xc, yc, e1, e2, lc, tlc_lo, t, w2min, g1, g2, th, kc, u2, omt;
   int npairs;
   RayLight light[2];
 };
@@ -284,7 +283,7 @@ __device__ __forceinline__ RayC ray_consts(const VecConst& v) {
   return {warp_uniform(v.xc), warp_uniform(v.yc),     warp_uniform(v.e1), warp_uniform(v.e2),
           warp_uniform(v.lc), warp_uniform(v.tlc_lo), warp_uniform(v.t),  warp_uniform(v.w2min),
           warp_uniform(v.g1), warp_uniform(v.g2),     warp_uniform(v.th), warp_uniform(v.kc),
-          warp_uniform(v.u2), warp_uniform(v.omt),    warp_uniform(v.den0), warp_uniform(v.npairs),
+          warp_uniform(v.u2), warp_uniform(v.omt),    warp_uniform(v.npairs),
           {ray_light(v.light[0]), ray_light(v.light[1])}};
 }
 

@@ -362,7 +362,6 @@ __global__ void k_setup(const __grid_constant__ Src src) {
       V->kc = 1.f - 0.5f * t;
       V->omt = 1.f - t;
       V->u2 = e2s;
-      V->den0 = 1.f + e2s;
       V->e1i = e1 * i1me2;
       V->e2i = e2 * i1me2;
     } else if (lane == 1 || lane == 2) {
@@ -798,11 +797,12 @@ __device__ __forceinline__ void ray_adj(const RayC& V, const Series<NP, true>& s
   }
   const T hr = fmaT(ur, Gr, fmaT(nui, Gi, sp<T>(1.f))), hi = fmaT(ur, Gi, ui * Gr);     // F
   const T tr = fmaT(ur, c1, nu2 * c2), ti = ui * c1;                                     // dF/dt / ln 2
-  // num = (t/2) F - (1 - t/2) G; F' v = num (v + eps) / |1 - u|^2, |1 - u|^2 = 1 + |u|^2 - 2 ur
-  // (conj(1 - u) v = v + eps |v|^2, |v| = 1)
+  // num = (t/2) F - (1 - t/2) G; F' v = num conj(1 - u) v / |1 - u|^2, both factors from the rounded 1 - u, so
+  // that its error enters once
   const T nr = fmaT(sp<T>(V.th), hr, sp<T>(-V.kc) * Gr), ni = fmaT(sp<T>(V.th), hi, sp<T>(-V.kc) * Gi);
-  const T idd = rcpT(sp<T>(V.den0) - ru);
-  const T er = (vr + sp<T>(V.e1)) * idd, ei = fmaT(sp<T>(2.f), vh, sp<T>(V.e2)) * idd;
+  const T dr = sp<T>(1.f) - ur;             // 1 - u = dr - i ui
+  const T idd = rcpT(fmaT(dr, dr, ui * ui)), ih = idd + idd;
+  const T er = vr * idd, ei = vh * ih;      // v / |1 - u|^2
   // lens equation with external shear, source at beta
   const T swr = S * wr, swi = S * wi, nswi = -swi;   // S w
   const T ar = fmaT(swr, hr, nswi * hi);
@@ -818,7 +818,8 @@ __device__ __forceinline__ void ray_adj(const RayC& V, const Series<NP, true>& s
   acc[A_THETAE] = acc[A_THETAE] + Zr;
   acc[A_T] = fmaT(lrho, Zr, fmaT(Cr, tr, fmaT(nCi, ti, acc[A_T])));
   // V = C F' v
-  const T Ur = fmaT(Cr, nr, nCi * ni), Ui = fmaT(Cr, ni, Ci * nr);
+  const T Nr = fmaT(nr, dr, ni * nui), Ni = fmaT(ni, dr, nr * ui);   // num conj(1 - u)
+  const T Ur = fmaT(Cr, Nr, nCi * Ni), Ui = fmaT(Cr, Ni, Ci * Nr);
   const T Vr = fmaT(Ur, er, -Ui * ei), Vi = fmaT(Ur, ei, Ui * er);
   const T t1 = sp<T>(V.omt) * Zr, nt1 = -t1;
   const T t2 = fmaT(sp<T>(-2.f * V.e1), Vi, fmaT(sp<T>(2.f * V.e2), Vr, Zi));
