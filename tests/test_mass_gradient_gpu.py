@@ -56,3 +56,12 @@ def test_ellipticity_enters_the_error_once(abi, eps):
     squared modulus formed as 1 + |u|^2 - 2 Re u has it to the second power."""
     err = _errors(abi, _rays(eps, int(100 * eps)))[0]
     assert np.percentile(err, 99) <= (8 + 6 / (1 - eps)) * 2.0 ** -24
+
+
+@pytest.mark.parametrize("eps", [0.2, 0.5, 0.8, 0.85])
+def test_slope_derivative_of_long_series(abi, eps):
+    """d/dgamma takes dF/dt, a sum of up to 90 terms here. Half of the rays
+    within three roundings and three that 1 / (1 - |eps|) enlarges, of the
+    entry: the sum of a long series adds none of its own."""
+    _, g, ref = _errors(abi, _rays(eps, 7 + int(100 * eps), gamma=(2.6, 2.9)))
+    assert np.median(np.abs(g[:, 1] - ref[:, 1]) / np.abs(ref[:, 1])) <= (3 + 3 / (1 - eps)) * 2.0 ** -24
