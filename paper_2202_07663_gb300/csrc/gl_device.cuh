@@ -93,7 +93,8 @@ struct __align__(16) VecConst {
   float omt;               // 1 - t
   float e1i, e2i;          // e1, e2 times 1 / (1 - |eps|^2)
   int order;               // written by k_order into slot p: the vector the ray kernels take p-th
-  float pad_[3];
+  float kn[2];             // b_n ln 2 / n of the lens light and the source
+  float pad_;
   LightC light[2];         // [0] lens light at theta, [1] source at beta
   // the series two terms at a time: (a_{2m+1}, a_{2m+2}, b_{2m+1}, b_{2m+2}), a_n = c_1 ... c_n and
   // b_n = d a_n / d t / ln 2, zero past the term count
@@ -266,7 +267,7 @@ __device__ __forceinline__ F2 grid_coord2(F2 n, float hh, float hl) { return fma
 // accumulators the adjoint then fitted three blocks per SM with spills
 // (k_ray_adj at 60 x 60, k = 2, B = 4096, three blocks per SM: 448.5 -> 428 us).
 struct RayLight {
-  float A, B2, C, x, y, c1, r2min, k1, I0;
+  float A, B2, C, x, y, c1, r2min, k1, I0, kn;
 };
 struct RayC {
   float xc, yc, e1, e2, lc, tlc_lo, t, w2min, g1, g2, th, kc, u2, omt;
@@ -275,16 +276,17 @@ struct RayC {
 };
 __device__ __forceinline__ float warp_uniform(float v) { return __shfl_sync(0xffffffffu, v, 0); }
 __device__ __forceinline__ int warp_uniform(int v) { return __shfl_sync(0xffffffffu, v, 0); }
-__device__ __forceinline__ RayLight ray_light(const LightC& l) {
+__device__ __forceinline__ RayLight ray_light(const LightC& l, float kn) {
   return {warp_uniform(l.A),  warp_uniform(l.B2),    warp_uniform(l.C),  warp_uniform(l.x), warp_uniform(l.y),
-          warp_uniform(l.c1), warp_uniform(l.r2min), warp_uniform(l.k1), warp_uniform(l.I0)};
+          warp_uniform(l.c1), warp_uniform(l.r2min), warp_uniform(l.k1), warp_uniform(l.I0),
+          warp_uniform(kn)};
 }
 __device__ __forceinline__ RayC ray_consts(const VecConst& v) {
   return {warp_uniform(v.xc), warp_uniform(v.yc),     warp_uniform(v.e1), warp_uniform(v.e2),
           warp_uniform(v.lc), warp_uniform(v.tlc_lo), warp_uniform(v.t),  warp_uniform(v.w2min),
           warp_uniform(v.g1), warp_uniform(v.g2),     warp_uniform(v.th), warp_uniform(v.kc),
           warp_uniform(v.u2), warp_uniform(v.omt),    warp_uniform(v.npairs),
-          {ray_light(v.light[0]), ray_light(v.light[1])}};
+          {ray_light(v.light[0], v.kn[0]), ray_light(v.light[1], v.kn[1])}};
 }
 
 // Elliptical Sersic at (px, py), generic in the ray type; the forward model,
