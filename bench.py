@@ -61,21 +61,23 @@ def flops_conv_pixel(K, grad, R=0):
 
 
 SERIES_TOL = 2e-8
+SERIES_T_MIN = 0.25
 NMAX = 128
 
 
 def series_terms(params: np.ndarray, adjoint: bool) -> np.ndarray:
     """Per-vector EPL series length, the rules the setup kernel applies:
     forward  smallest N >= 0 with |a_(N+1)| f^(N+1) / (1 - f max(1, c_(N+2))) <= tol,
-             a_n = c_1 ... c_n, c_k = (2k - 2 + t) / (2k + 2 - t), t = gamma - 1,
+             a_n = c_1 ... c_n, c_k = (2k - 2 + t) / (2k + 2 - t), t = gamma - 1 (|t| >= 0.25 in c_1),
     adjoint  the same N, at least 1."""
     p = params.astype(np.float64)
     f = np.hypot(p[:, 2], p[:, 3])[:, None]
     t = (p[:, 1] - 1.0)[:, None]
     k = np.arange(1, NMAX + 2)[None, :]
-    c = (2 * k - 2 + t) / (2 * k + 2 - t)                    # c_1 .. c_(NMAX+1)
+    c = np.abs((2 * k - 2 + t) / (2 * k + 2 - t))            # |c_1| .. |c_(NMAX+1)|
+    c[:, :1] = np.maximum(c[:, :1], SERIES_T_MIN / (4 - t))
     with np.errstate(divide="ignore"):
-        la = np.cumsum(np.log(np.abs(c)), axis=1)             # log|a_1| .. log|a_(NMAX+1)|
+        la = np.cumsum(np.log(c), axis=1)            # log|a_1| .. log|a_(NMAX+1)|
         lf = np.where(f > 0, np.log(np.maximum(f, 1e-300)), -1e300)
     N = np.arange(0, NMAX + 1)[None, :]
     kk = N + 2

@@ -227,9 +227,13 @@ __device__ void setup_fp64_part(const Src& src, int item, int part) {
 // a bound on |F - F_N| (|c_k| decreases toward 1 for k >= 2, so the tail after
 // a_{N+1} is at most a geometric series of ratio f max(1, c_{N+2})). The
 // adjoint uses the same N (at least 1): its dF/du comes from F and h_1 in
-// closed form, and the tail of dF/dt exceeds that of F only by a logarithmic
-// factor.
+// closed form. d a_n / d t = a_n (1/t + O(log n)): every a_n has the factor t
+// of c_1 = t / (4 - t), its derivative has not, so toward t = 0 (gamma = 1) the
+// tail of dF/dt is 1/|t| times F's. The test therefore takes |t| of c_1 as at
+// least SERIES_T_MIN, which bounds the tail of dF/dt by about SERIES_TOL (1 /
+// SERIES_T_MIN + log N), 2e-7, and leaves N as F needs it from there on.
 constexpr double SERIES_TOL = 2e-8;
+constexpr float SERIES_T_MIN = 0.25f;
 
 __device__ __forceinline__ float series_coef(int k, float t) { return (2.f * k - 2.f + t) / (2.f * k + 2.f - t); }
 __device__ __forceinline__ float series_dcoef(int k, float t) {   // d c_k / d t = 4k / (2k + 2 - t)^2
@@ -245,7 +249,10 @@ template <int NC>
 __device__ __forceinline__ int term_count(int lane, float t, float f, float lf, float ltol) {
   float la[NC];
 #pragma unroll
-  for (int m = 0; m < NC; ++m) la[m] = logf(fabsf(series_coef(lane + 1 + 32 * m, t)));
+  for (int m = 0; m < NC; ++m) {
+    const float c = fabsf(series_coef(lane + 1 + 32 * m, t));
+    la[m] = logf(lane + m == 0 ? fmaxf(c, SERIES_T_MIN / (4.f - t)) : c);
+  }
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
 #pragma unroll

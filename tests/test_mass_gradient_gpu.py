@@ -65,3 +65,12 @@ def test_slope_derivative_of_long_series(abi, eps):
     entry: the sum of a long series adds none of its own."""
     _, g, ref = _errors(abi, _rays(eps, 7 + int(100 * eps), gamma=(2.6, 2.9)))
     assert np.median(np.abs(g[:, 1] - ref[:, 1]) / np.abs(ref[:, 1])) <= (3 + 3 / (1 - eps)) * 2.0 ** -24
+
+
+@pytest.mark.parametrize("gamma", [1.0, 1.001, 1.1, 1.26, 0.9])
+@pytest.mark.parametrize("eps", [0.05, 0.3, 0.6])
+def test_slope_derivative_near_the_isothermal_limit(abi, eps, gamma):
+    """At gamma = 1 every coefficient of F vanishes and its derivative does
+    not: the series is as long as dF/dt needs. The bound of the long series."""
+    _, g, ref = _errors(abi, _rays(eps, 11, gamma=(gamma, gamma)))
+    assert np.median(np.abs(g[:, 1] - ref[:, 1]) / np.abs(ref[:, 1])) <= (3 + 3 / (1 - eps)) * 2.0 ** -24
