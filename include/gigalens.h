@@ -148,7 +148,11 @@ int gl_system_psf_rank(const gl_system* sys);
 int gl_system_destroy(gl_system* sys);
 
 /* Pre-size the system's scratch for batches of up to B vectors so that later
- * calls with B' <= B allocate nothing. */
+ * calls with any B' <= B allocate nothing and leave its addresses as they are
+ * (a captured call keeps them). It covers gl_loglik, gl_loglik_grad,
+ * gl_loglik_grad_f32, gl_simulate and the system's part of a grouped call; the
+ * host-buffer and the profiled calls hold more and grow it at their first call
+ * of a size. */
 int gl_system_reserve(gl_system* sys, int B);
 
 /* Device bytes the system's scratch needs for a batch of B vectors. */

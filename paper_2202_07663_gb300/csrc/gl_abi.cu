@@ -537,16 +537,7 @@ int gl_system_reserve(gl_system* s, int B) {
   if (B < 0 || B > (1 << 24)) return fail(GL_ERR_INVALID_ARG, "B = %d", B);
   int rc = check_device(s);
   if (rc != GL_OK) return rc;
-  // partial need is largest at small B (more tiles per vector); take the max over B' <= B
-  long long need = 0;
-  for (int b : {1, 2, 4, 8, 16, 32, 64, 128, 256, 512, 1024, 2048, B}) {
-    if (b > B || b < 1) continue;
-    int nt, tp;
-    long long p;
-    partial_need(s, b, &nt, &tp, &p);
-    need = p > need ? p : need;
-  }
-  return ensure_scratch(s, B, need);
+  return ensure_scratch(s, B, gl::max_tiles(B, s->H, s->W, s->k) * gl::NACC);
 }
 
 int gl_loglik(gl_system* s, const float* params, int B, double* loglik_out, double* chi2_out, void* stream) {

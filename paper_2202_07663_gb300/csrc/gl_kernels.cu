@@ -2369,17 +2369,25 @@ static double ray_kernel_cost(double items, double px, double slots, double tail
   return px * (full + part + tail);
 }
 
+// The most tiles a vector of an H x W image may have by its size, and the most
+// that all vectors of a call may have together unless each has just one (past
+// sixteen waves of the adjoint a finer tiling evens out nothing).
+static long long tiles_by_size(int H, int W, int k) {
+  const long long HW = (long long)H * W, rays = HW * k * k;
+  const long long by_pixels = (HW + 2 * ADJ_THREADS - 1) / (2 * ADJ_THREADS);
+  const long long by_rays = (rays + 4 * ADJ_THREADS - 1) / (4 * ADJ_THREADS);
+  return by_rays < by_pixels ? by_rays : by_pixels;
+}
+static long long tiles_by_waves() { return 16LL * num_sms() * ADJ_BLOCKS_PER_SM; }
+
 static TilePlan plan_rays(int B, int H, int W, int k) {
   constexpr double TILE_RAYS = 400.0, TAIL = 0.25;
   const int HW = H * W;
   TilePlan best{1, HW};
   if (B <= 0 || HW <= 0) return best;
-  const long long rays = (long long)HW * k * k;
-  long long max_nt = (HW + 2 * ADJ_THREADS - 1) / (2 * ADJ_THREADS);
-  const long long by_rays = (rays + 4 * ADJ_THREADS - 1) / (4 * ADJ_THREADS);
-  if (by_rays < max_nt) max_nt = by_rays;
+  long long max_nt = tiles_by_size(H, W, k);
   const double sms = num_sms(), fwd_slots = sms * fwd_blocks_per_sm(), adj_slots = sms * ADJ_BLOCKS_PER_SM;
-  const long long by_waves = (long long)(16.0 * adj_slots / B);   // past sixteen waves a finer tiling evens out nothing
+  const long long by_waves = tiles_by_waves() / B;
   if (by_waves < max_nt) max_nt = by_waves;
   if (max_nt < 1) max_nt = 1;
   const double tail = B < sms ? 0.0 : TAIL;
@@ -2403,6 +2411,15 @@ void plan_tiles(int B, int H, int W, int k, int* ntiles, int* tile_pix) {
   const TilePlan p = plan_rays(B, H, W, k);
   *ntiles = p.ntiles;
   *tile_pix = p.tile_pix;
+}
+
+// B' ntiles(B') is not monotone in B' and jumps by whole tiles per vector, so
+// the bound comes from the plan's two limits, not from samples of it.
+long long max_tiles(int B, int H, int W, int k) {
+  if (B <= 0) return 0;
+  const long long by_size = B * tiles_by_size(H, W, k), by_waves = tiles_by_waves();
+  const long long n = by_size < by_waves ? by_size : by_waves;
+  return n > B ? n : B;
 }
 
 // Blocks of a convolution kernel resident on the whole GPU at a dynamic

@@ -63,6 +63,8 @@ struct ConvRun {
 
 // Split each vector's detector pixels into ray tiles for a batch of B.
 void plan_tiles(int B, int H, int W, int k, int* ntiles, int* tile_pix);
+// At least the tiles of any call of 1 .. B vectors, over all of its vectors.
+long long max_tiles(int B, int H, int W, int k);
 
 // One segment, passed by value.
 cudaError_t launch_one(const Seg& s, int mode, cudaStream_t st, Hooks* hooks);
