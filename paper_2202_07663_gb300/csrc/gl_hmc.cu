@@ -94,9 +94,10 @@ __global__ void k_affine(int B, int d, const double* __restrict__ x, const doubl
 }
 
 // out[b][j] = (float)(scale[b] rows[b][j]), the product in FP64.
-__global__ void k_scale_rows_f32(int n, int d, const float* __restrict__ scale, size_t stride,
+__global__ void k_scale_rows_f32(unsigned n, unsigned d, const float* __restrict__ scale, size_t stride,
                                  const double* __restrict__ rows, float* __restrict__ out) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
+  // unsigned: n < 2^31 and a step of at most 2^20 stay below 2^32, and the division stays 32-bit
+  for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
     out[i] = float(double(scale[size_t(i / d) * stride]) * rows[i]);
 }
 
@@ -293,7 +294,8 @@ int gl_scale_rows_f32(int B, int d, const float* scale, size_t scale_stride, con
   gl::Hooks* h = gl_internal::hooks();
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   h->before(GL_K_OTHER, st);
-  k_scale_rows_f32<<<grid_for((long long)B * d, 256), 256, 0, st>>>(B * d, d, scale, scale_stride, rows, out);
+  k_scale_rows_f32<<<grid_for((long long)B * d, 256), 256, 0, st>>>(unsigned(B) * unsigned(d), unsigned(d), scale,
+                                                                     scale_stride, rows, out);
   cudaError_t e = h->after(GL_K_OTHER, st);
   return e == cudaSuccess ? GL_OK : gl_internal::cuda_error(e, "k_scale_rows_f32");
 }

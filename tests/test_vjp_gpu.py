@@ -127,3 +127,23 @@ def test_dispatch_mode_sees_the_product(setup):
         (out,) = torch.autograd.grad(ll, p, grad_outputs=w)
     assert any(name.startswith("aten.mul") for name in seen)
     assert torch.equal(out, _expression(w, s.loglik_grad(p0)[1]))
+
+
+def test_scaled_rows_up_to_the_largest_product(setup):
+    """B d = 2^31 - 4096, where a 32-bit signed index would step past its range:
+    the first and last rows scaled, nothing else touched (26 GB)."""
+    from paper_2202_07663_gb300 import abi
+    B, d = (1 << 19) - 1, 4096
+    if torch.cuda.mem_get_info()[0] < 40 << 30:
+        pytest.skip("needs 40 GB free")
+    rows = torch.zeros(B, d, dtype=torch.float64, device="cuda")
+    out = torch.full((B, d), 7.0, dtype=torch.float32, device="cuda")
+    rows[0], rows[-1] = 1.0, torch.arange(d, dtype=torch.float64, device="cuda")
+    scale = torch.full((B,), 2.0, device="cuda")
+    scale[-1] = 3.0
+    abi.gl_scale_rows_f32(B, d, scale.data_ptr(), 1, rows.data_ptr(), out.data_ptr(), abi._stream_ptr(out.device))
+    assert torch.equal(out[0], torch.full((d,), 2.0, device="cuda"))
+    assert torch.equal(out[-1], 3.0 * torch.arange(d, dtype=torch.float32, device="cuda"))
+    assert int(torch.count_nonzero(out)) == d + d - 1
+    del rows, out
+    torch.cuda.empty_cache()
