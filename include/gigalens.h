@@ -250,7 +250,8 @@ int gl_loglik_grad_grouped(gl_system* const* systems, const float* const* params
  * buffer, per-tile gradient partials) lives in one static device array of
  * 32 MiB (33,554,432 bytes), which every GPU that loads
  * the library holds until the process exits. A batch whose scratch does not
- * fit is rejected with GL_ERR_INVALID_ARG before anything is launched (about
+ * fit even with one ray tile per vector (it takes fewer tiles near the limit)
+ * is rejected with GL_ERR_INVALID_ARG before anything is launched (about
  * 2,100 vectors of a 60 x 60 image; scratch per vector is 4*H*W + 1,232
  * bytes plus 192 bytes per ray tile, gl_system_scratch_bytes(sys, B) / B).
  *

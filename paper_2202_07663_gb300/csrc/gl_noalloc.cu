@@ -55,7 +55,14 @@ int gl_loglik_grad_noalloc(gl_system* sys, const float* params, int B, double* l
   gl::Seg g = gl_internal::seg_without_scratch(sys, params, B);
   const size_t vc_bytes = align256(sizeof(gl::VecConst) * size_t(B));
   const size_t work_bytes = align256(sizeof(float) * size_t(B) * g.H * g.W);
-  const size_t part_bytes = align256(sizeof(double) * size_t(B) * g.ntiles * gl::NACC);
+  // the tile plan serves speed alone: where its partials do not fit beside the rest, as many tiles as do
+  const size_t per_tile = sizeof(double) * size_t(B) * gl::NACC, rest = vc_bytes + work_bytes;
+  if (rest + align256(per_tile * g.ntiles) > kNoAllocScratchBytes && rest + align256(per_tile) <= kNoAllocScratchBytes) {
+    const long long HW = (long long)g.H * g.W, n = (kNoAllocScratchBytes - rest) / per_tile;
+    g.tile_pix = int((HW + n - 1) / n);
+    g.ntiles = int((HW + g.tile_pix - 1) / g.tile_pix);
+  }
+  const size_t part_bytes = align256(per_tile * g.ntiles);
   const size_t need = vc_bytes + work_bytes + part_bytes;
   if (need > kNoAllocScratchBytes) {
     char msg[200];
