@@ -212,22 +212,15 @@ __device__ __forceinline__ F2 operator-(F2 a) {
 }
 
 template <class T> __device__ __forceinline__ T sp(float a);
-template <> __device__ __forceinline__ float sp<float>(float a) { return a; }
 template <> __device__ __forceinline__ F2 sp<F2>(float a) { return {make_float2(a, a)}; }
 
-__device__ __forceinline__ float fmaT(float a, float b, float c) { return fmaf(a, b, c); }
 __device__ __forceinline__ F2 fmaT(F2 a, F2 b, F2 c) { return {__ffma2_rn(a.v, b.v, c.v)}; }
-__device__ __forceinline__ float ex2T(float a) { return ex2(a); }
 __device__ __forceinline__ F2 ex2T(F2 a) { return {make_float2(ex2(a.v.x), ex2(a.v.y))}; }
-__device__ __forceinline__ float lg2T(float a) { return lg2(a); }
 __device__ __forceinline__ F2 lg2T(F2 a) { return {make_float2(lg2(a.v.x), lg2(a.v.y))}; }
-__device__ __forceinline__ float rcpT(float a) { return rcp(a); }
 __device__ __forceinline__ F2 rcpT(F2 a) { return {make_float2(rcp(a.v.x), rcp(a.v.y))}; }
-__device__ __forceinline__ float maxT(float a, float b) { return fmaxf(a, b); }
 __device__ __forceinline__ F2 maxT(F2 a, F2 b) { return {make_float2(fmaxf(a.v.x, b.v.x), fmaxf(a.v.y, b.v.y))}; }
 // v where a >= b, else 0, by selection (a 0/1 factor would be one more
 // instruction of the FP32 pipe)
-__device__ __forceinline__ float where_ge(float a, float b, float v) { return a >= b ? v : 0.f; }
 __device__ __forceinline__ F2 where_ge(F2 a, F2 b, F2 v) {
   return {make_float2(a.v.x >= b.v.x ? v.v.x : 0.f, a.v.y >= b.v.y ? v.v.y : 0.f)};
 }
@@ -238,15 +231,8 @@ __device__ __forceinline__ F2 where_ge(F2 a, F2 b, F2 v) {
 // Sersic profile like a change of its parameters. One correction step: with
 // y0 = lg2.approx(x), log2 x = y0 + log2(x 2^-y0) and x 2^-y0 - 1 (one FMA on
 // ex2.approx(-y0), whose mean error is -8e-9) is ln 2 times that remainder
-// to first order (the remainder is ~1e-7, its square negligible).
-__device__ __forceinline__ float lg2c(float x) {
-  const float y0 = lg2(x);
-  const float d = fmaf(x, ex2(-y0), -1.f);
-  return fmaf(d, 1.44269504088896341f, y0);
-}
-__device__ __forceinline__ float lg2cT(float a) { return lg2c(a); }
-// The same correction on a packed pair: per lane the arithmetic of lg2c (the
-// two FMAs as one packed FMA each).
+// to first order (the remainder is ~1e-7, its square negligible). The two
+// FMAs as one packed FMA each.
 __device__ __forceinline__ F2 lg2cT(F2 a) {
   const float y0x = lg2(a.v.x), y0y = lg2(a.v.y);
   const F2 e = {make_float2(ex2(-y0x), ex2(-y0y))};
@@ -289,7 +275,7 @@ __device__ __forceinline__ RayC ray_consts(const VecConst& v) {
           {ray_light(v.light[0], v.kn[0]), ray_light(v.light[1], v.kn[1])}};
 }
 
-// Elliptical Sersic at (px, py), generic in the ray type; the forward model,
+// Elliptical Sersic at (px, py) of a packed pair of rays; the forward model,
 // so its log2 is the unbiased one (log L sums the model over every pixel).
 // The terms of dy alone come first: the ray loops step x innermost, so the
 // compiler can keep the lens light's out of the inner loop.
@@ -334,7 +320,7 @@ struct Series<0, ADJ> {
   __device__ __forceinline__ float4 pair(int m) const { return ser[m]; }
 };
 
-// Source-plane position of a ray, generic in the ray type: beta = theta -
+// Source-plane position of a packed pair of rays: beta = theta -
 // alpha_EPL - alpha_shear. A ray inside rho < 1e-6 arcsec gets zero EPL
 // deflection (mask), computed without a branch so pairs stay in lockstep.
 // G = sum_{n<N} a_{n+1} u^n by Horner's rule; the two highest terms start the

@@ -707,8 +707,7 @@ constexpr float B_N = 1.9992f;   // b_n / n = 1.9992 - 0.3271 / n
 // every ray of a vector shares (A, B, C and their derivatives in e1, e2), so
 // k_final forms them once per vector instead of each ray. With POS also
 // returns Gx = gq (A dx + B dy), Gy = gq (B dx + C dy) (B = B2 / 2): the ray's
-// position derivative over -(b_n / n) I0. Generic in the ray type (float or a
-// packed pair).
+// position derivative over -(b_n / n) I0. T: a packed pair of rays.
 template <bool POS, class T>
 __device__ __forceinline__ void light_adj(const RayLight& L, T px, T py, T g, T* acc, T& Gx, T& Gy) {
   const T dx = px - sp<T>(L.x), dy = py - sp<T>(L.y);
@@ -2648,20 +2647,13 @@ static cudaError_t launch_order(const Src&, int, cudaStream_t) { return cudaErro
 
 template <class Src>
 static cudaError_t run_rays(const Src& src, int nvec, int nray, bool fwd, bool adj_final, cudaStream_t st,
-                            Hooks* hooks, bool persistent, bool one_tile = false, bool fwd_rays = true) {
-  const int sms = num_sms();
+                            Hooks* hooks, bool one_tile = false, bool fwd_rays = true) {
   cudaError_t e;
   const int vthreads = SETUP_THREADS, wpb = vthreads / 32 - 2;
-  int sgrid = (nvec + wpb - 1) / wpb;
-  int fgrid = (nvec + FINAL1_THREADS - 1) / FINAL1_THREADS;
-  int wgrid = (nvec + FINAL_THREADS / 32 - 1) / (FINAL_THREADS / 32);
-  int rgrid = nray;
-  if (persistent) {
-    sgrid = sgrid < sms * 4 ? sgrid : sms * 4;
-    fgrid = fgrid < sms * 4 ? fgrid : sms * 4;
-    wgrid = wgrid < sms * 4 ? wgrid : sms * 4;
-    rgrid = rgrid < sms * 4 ? rgrid : sms * 4;
-  }
+  const int sgrid = (nvec + wpb - 1) / wpb;
+  const int fgrid = (nvec + FINAL1_THREADS - 1) / FINAL1_THREADS;
+  const int wgrid = (nvec + FINAL_THREADS / 32 - 1) / (FINAL_THREADS / 32);
+  const int rgrid = nray;
   if (fwd) {
     if (takes_order(src)) {
       for (int stage = nvec <= ORDER_OWN_KEYS ? 1 : 0; stage < 2; ++stage) {   // k_keys, k_order
@@ -2731,17 +2723,17 @@ cudaError_t launch_one(const Seg& s0, int mode, cudaStream_t st, Hooks* hooks) {
   // MODE_CORR already holds the vectors' d log L / d M
   s.ray_order = mode != MODE_CORR && ray_order_pays(s) ? 1 : 0;
   OneSeg src{s};
-  cudaError_t e = run_rays(src, s.B, s.B * s.ntiles, true, false, st, hooks, false, false, mode != MODE_CORR);
+  cudaError_t e = run_rays(src, s.B, s.B * s.ntiles, true, false, st, hooks, false, mode != MODE_CORR);
   if (e != cudaSuccess) return e;
   if ((e = launch_conv_single(src, mode, st, hooks)) != cudaSuccess) return e;
   if (mode != MODE_GRAD && mode != MODE_CORR) return cudaSuccess;
-  return run_rays(src, s.B, s.B * s.ntiles, false, true, st, hooks, false, s.ntiles == 1);
+  return run_rays(src, s.B, s.B * s.ntiles, false, true, st, hooks, s.ntiles == 1);
 }
 
 cudaError_t launch_basis(const Seg& s, cudaStream_t st, Hooks* hooks) {
   if (s.B <= 0) return cudaSuccess;
   OneSeg src{s};
-  cudaError_t e = run_rays(src, s.B, s.B * s.ntiles, true, false, st, hooks, false, false, false);   // setup
+  cudaError_t e = run_rays(src, s.B, s.B * s.ntiles, true, false, st, hooks, false, false);   // setup
   if (e != cudaSuccess) return e;
   hooks->before(GL_K_RAY_FWD, st);
   if ((e = launch_pdl(k_ray_fwd_basis<OneSeg>, unsigned(s.B * s.ntiles), FWD_THREADS, 0, st, src)) != cudaSuccess)
@@ -2760,7 +2752,7 @@ cudaError_t launch_table(const Seg* d_segs, int nseg, int vec_total, int ray_tot
                          int mode, cudaStream_t st, Hooks* hooks) {
   if (vec_total <= 0) return cudaSuccess;
   SegTable src{d_segs, nseg, vec_total, ray_total, 0, nseg, vec_total};
-  cudaError_t e = run_rays(src, vec_total, ray_total, true, false, st, hooks, false);
+  cudaError_t e = run_rays(src, vec_total, ray_total, true, false, st, hooks);
   if (e != cudaSuccess) return e;
   for (int i = 0; i < nconv; ++i) {
     SegTable cs = src;
@@ -2774,7 +2766,7 @@ cudaError_t launch_table(const Seg* d_segs, int nseg, int vec_total, int ray_tot
     if ((e = hooks->after(GL_K_CONV, st)) != cudaSuccess) return e;
   }
   if (mode != MODE_GRAD) return cudaSuccess;
-  return run_rays(src, vec_total, ray_total, false, true, st, hooks, false);
+  return run_rays(src, vec_total, ray_total, false, true, st, hooks);
 }
 
 // Grouped launch whose counts live in device memory: fixed persistent grids,
