@@ -188,9 +188,8 @@ int gl_loglik(gl_system* sys, const float* params, int B, double* loglik_out, do
 /*
  * gl_loglik_grad - gl_loglik plus d log L / d params (Sec. 2.2), computed
  * by a hand-written adjoint: the pixel adjoint is correlated with the PSF
- * and spread over the k x k subpixels, then every ray is recomputed and its
- * forward-mode derivatives are contracted with that adjoint. No ray position
- * is stored.
+ * and spread over the k x k subpixels, then every ray is recomputed and that
+ * adjoint is carried back through it. No ray position is stored.
  *
  *  grad_out    device float64 [B, 22], same order as params.
  */
@@ -599,7 +598,7 @@ enum gl_kernel_kind {
   GL_K_SETUP = 0,    /* per-vector constants */
   GL_K_RAY_FWD = 1,  /* ray shooting + lights + k x k binning */
   GL_K_CONV = 2,     /* PSF convolution + likelihood (+ pixel adjoint) */
-  GL_K_RAY_ADJ = 3,  /* recomputed rays + forward-mode derivatives */
+  GL_K_RAY_ADJ = 3,  /* recomputed rays, the subpixel adjoint carried back through each */
   GL_K_FINAL = 4,    /* per-vector gradient reduction */
   GL_K_OTHER = 5,
   GL_K_ORDER = 6     /* order of a call's vectors, longest EPL series first:

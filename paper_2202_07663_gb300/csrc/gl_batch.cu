@@ -208,8 +208,7 @@ int gl_batcher_run(gl_batcher* b, gl_system* const* systems, const float* const*
   if (nonempty == 1) {
     // One segment (the common case of a lightly loaded server): the launch
     // sequence of a single-system call, tuned for its batch size (tile plan,
-    // adjoint blocks per SM, small-batch convolution), on its share of the
-    // arena; no table, no graph.
+    // small-batch convolution), on its share of the arena; no table, no graph.
     gl::Seg g;
     for (int c = 0; c < gl::N_CONV_CLASSES; ++c)
       if (!by_class[c].empty()) g = by_class[c][0];

@@ -400,7 +400,8 @@ __global__ void k_setup(const __grid_constant__ Src src) {
 
 // Slots of a call's vectors, longest EPL series first (the order the ray
 // kernels then take them in). A ray's cost grows with the vector's series
-// terms N (331 + 14 N flops in the adjoint, 90 + 7 N in the forward), and a
+// terms N (199 + 11 N flops in the adjoint, 200 + 14 N past twelve terms, 85 +
+// 7 N in the forward), and a
 // batch drawn from a prior mixes short and long series; with the heaviest
 // vectors' blocks in the first waves the last waves hold the lightest
 // (longest-processing-time first). The order is fixed before k_setup, so its
@@ -413,13 +414,14 @@ __global__ void k_setup(const __grid_constant__ Src src) {
 // the vector each slot holds. Above ORDER_OWN_KEYS vectors k_keys forms the
 // keys over many blocks (one block reading every vector's row of parameters
 // waits on one SM's scattered loads: 11.8 us at B = 4096); up to it, one
-// vector per thread, k_order forms them itself and a launch is saved (B =
-// 300: 21 -> 14 us with its launch between events; the call's launches 7 -> 6). k_order, one block, is a counting
-// sort: each warp counts its vectors per key in a row of its own (shared-
-// memory atomics that never meet another warp's: a batch's keys crowd into
-// a few values, and one counter per key for the whole block would make the
-// warps wait on each other), a block-wide scan over (key from the largest down, warp)
-// turns the counts into first slots, and each warp hands out its slots.
+// vector per thread, k_order forms them itself and a launch is saved (B = 300:
+// 21 -> 14 us with its launch between events; the call's launches 7 -> 6).
+// k_order, one block, is a counting sort: each warp counts its vectors per key
+// in a row of its own (shared-memory atomics that never meet another warp's: a
+// batch's keys crowd into a few values, and one counter per key for the whole
+// block would make the warps wait on each other), a block-wide scan over (key
+// from the largest down, warp) turns the counts into first slots, and each warp
+// hands out its slots.
 // Within one (key, warp) the slots follow the order the warp's atomics are
 // served in; results do not depend on the slots. k_setup reads its slot's
 // vector from slot[] and keeps it in VecConst::order for the later kernels.
@@ -756,13 +758,16 @@ __device__ __forceinline__ void light_adj(const RayLight& L, T px, T py, T g, T*
 // so the centre needs only the sums of q, and eps adds one per-vector term
 // (both in k_final). dF/du = [(t/2) F - (1 - t/2) G] / (1 - u), G = (F - 1) / u
 // (Gauss contiguous relation), without a cancellation. The kernel is bound by
-// the FP32 pipe (71% busy) and its latency, and per ray this is about two
+// the FP32 pipe (three quarters busy) and its latency, and per ray this is about two
 // thirds of the arithmetic of forming each parameter's d alpha: k_ray_adj at
 // 60 x 60, k = 2, B = 4096, 607 -> 459 us; with the signs on the integer pipe
 // and float-stepped grid indices 448, the constants warp-uniform (RayC) and
 // four blocks per SM 406, the series two terms a step and pixels stepped
-// without divisions 388, the series in straight-line code (Series) 367. The lens light in a loop of its own, so that its
-// eight accumulators are not live with the others: 412.
+// without divisions 388, the series in straight-line code (Series) 367. What
+// keeps the error of forming each d alpha costs 13 of that: 1 / (1 - u) from the
+// rounded 1 - u, long series' dF/dt in Horner's form, the index's term per ray:
+// 380. The lens light in a loop of its own, so that its eight accumulators are
+// not live with the others: 412 against 388.
 //
 // F and the source position stay in Horner's form: next to the source's centre
 // the gradient follows the last bits of the position (a cusp's slope), and
@@ -868,10 +873,10 @@ __device__ __forceinline__ void ray_adj(const RayC& V, const Series<NP, true>& s
 }
 
 // Block size and resident blocks per SM of the adjoint kernel. With the series
-// in straight-line code, three blocks of 128 threads (168 registers, no
+// in straight-line code, three blocks of 128 threads (166 registers, no
 // spills) against four (128, some 100 bytes of spills in each length's code):
 // 367 and 378 us at 60 x 60, k = 2, B = 4096; 473 and 489 us at 100 x 100, k = 4,
-// B = 512. 160 x 3 393, 96 x 5 394, 192 x 2 389, 64 x 7 384, 64 x 6 376 us.
+// B = 512 (three now 380 and 495). 160 x 3 393, 96 x 5 394, 192 x 2 389, 64 x 7 384, 64 x 6 376 us.
 constexpr int ADJ_THREADS = 128;
 constexpr int ADJ_BLOCKS_PER_SM = 3;
 
@@ -1150,10 +1155,11 @@ __device__ __forceinline__ float pixel_terms(const Seg& s, int p, float M, float
 // of float4 per row, so the 8 lanes of each 128-bit shared-memory phase hit
 // 8 distinct bank groups. The sides 11 and 21 are compiled whole; any other
 // odd side runs in groups of 16 taps and one of K mod 16 (compiled for each
-// remainder), which keeps the loads at one float4 per 32 FMAs or fewer. The
-// column strips that those sides took before read every input value through
-// a scalar load: 61 x 59, K = 13, 200 vectors 131 -> 26 us; 108 x 108,
-// K = 17, one vector 508 -> 19.5 us (with its row bands).
+// remainder): 12 float4 loads for a group's 256 FMAs (20 with mirrored rows), 5
+// for the 16 of a remainder of one tap. The column strips that those sides
+// took before read every input value through a scalar load: 61 x 59, K = 13,
+// 200 vectors 131 -> 26 us; 108 x 108, K = 17, one vector 508 -> 19.5 us (with
+// its row bands).
 //
 // mirror: the PSF's rows are the same from the top and from the bottom (any
 // profile sampled on a centred grid; gl_system_create checks every value), so
@@ -2356,8 +2362,8 @@ static int fwd_blocks_per_sm() {
 // adjoint by tile count: 300 prior draws of 80 x 80 2: 119, 3: 106, 4: 103.5, 6:
 // 104, 8: 106, 12: 114 us; 50 vectors near one mode 6: 29.8, 9: 30.3, 12: 30.0, 15:
 // 32.3; 512 vectors of 100 x 100, k = 4, 1: 797, 2: 683, 4: 682, 8: 679, 12: 699. A
-// larger count must gain 1.5%. Tiles keep at least one step of a block (two
-// pixels a thread) and four rays a thread.
+// larger count must gain 1.5%. There are at most as many tiles as steps of a
+// block (two pixels a thread) and as 512 rays (four a thread), both rounded up.
 struct TilePlan {
   int ntiles, tile_pix;
 };
@@ -2439,7 +2445,7 @@ static cudaError_t conv_resident(size_t smem, int* resident) {
   return cudaSuccess;
 }
 
-// Launch with programmatic stream serialization (see pdl_begin): the kernel
+// Launch with programmatic stream serialization (see PdlScope): the kernel
 // may be scheduled while its predecessor in the stream drains.
 template <typename... KArgs, typename... Args>
 static cudaError_t launch_pdl(void (*kern)(KArgs...), unsigned grid, unsigned block, size_t smem, cudaStream_t st,

@@ -57,7 +57,8 @@ int gl_loglik_grad_noalloc(gl_system* sys, const float* params, int B, double* l
   const size_t work_bytes = align256(sizeof(float) * size_t(B) * g.H * g.W);
   // the tile plan serves speed alone: where its partials do not fit beside the rest, as many tiles as do
   const size_t per_tile = sizeof(double) * size_t(B) * gl::NACC, rest = vc_bytes + work_bytes;
-  if (rest + align256(per_tile * g.ntiles) > kNoAllocScratchBytes && rest + align256(per_tile) <= kNoAllocScratchBytes) {
+  if (rest + align256(per_tile * g.ntiles) > kNoAllocScratchBytes &&
+      rest + align256(per_tile) <= kNoAllocScratchBytes) {
     const long long HW = (long long)g.H * g.W, n = (kNoAllocScratchBytes - rest) / per_tile;
     g.tile_pix = int((HW + n - 1) / n);
     g.ntiles = int((HW + g.tile_pix - 1) / g.tile_pix);
