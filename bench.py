@@ -95,7 +95,7 @@ MUFU_RAY_ADJ = 12   # ex2/lg2/rcp per ray in the adjoint: EPL 4 (lg2, ex2, two r
 # DRAM bytes per launch of k_ray_adj from one ncu capture, keyed by workload
 # and the kernel source it was taken on (sha256 prefix of gl_kernels.cu +
 # gl_device.cuh); any other source reports null traffic until it is captured again.
-TRAFFIC = {("multistart-60x60-k2-psf11-B4096", "eee27ee73810b968"): 64.142e6}
+TRAFFIC = {("multistart-60x60-k2-psf11-B4096", "1d80f4572fe3c87c"): 64.455e6}
 
 
 def kernel_source_hash() -> str:
