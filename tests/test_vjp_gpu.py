@@ -91,7 +91,8 @@ def test_incoming_gradient_whose_memory_holds_its_negative(setup):
     (go,) = torch.autograd.grad(value, ll, retain_graph=True)
     (out,) = torch.autograd.grad(value, p)
     assert torch.equal(out, _expression(-z.real, g)) and torch.equal(out, _expression(go, g))
-    (out,) = torch.autograd.grad(hmc.loglik(p, s), p, grad_outputs=torch._efficientzerotensor((len(p0),), device="cuda"))
+    zero = torch._efficientzerotensor((len(p0),), device="cuda")
+    (out,) = torch.autograd.grad(hmc.loglik(p, s), p, grad_outputs=zero)
     assert torch.equal(out, torch.zeros_like(out))
 
 
